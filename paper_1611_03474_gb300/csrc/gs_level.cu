@@ -426,36 +426,23 @@ int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const
 }
 
 // ---------------------------------------------------------------- estimation
-// Truncated SVD bounds of section 2.2.2, templated on the arithmetic type.
+// Truncated SVD bounds of section 2.2.2: FP32 one thread per cube, FP64
+// (further down) four lanes per cube.
 
 template <typename T> __device__ __forceinline__ T t_sqrt(T x);
 template <> __device__ __forceinline__ double t_sqrt<double>(double x) { return sqrt(x); }
 template <> __device__ __forceinline__ float t_sqrt<float>(float x) { return sqrtf(x); }
 template <typename T> __device__ __forceinline__ T t_abs(T x) { return x < T(0) ? -x : x; }
-template <typename T> struct Eps;
 // Jacobi rotation zeroing the inner product ga of two rows with squared
-// norms al, be; false when the rows are already orthogonal to within Eps
-template <typename T> __device__ __forceinline__ bool jac_rot(T al, T be, T ga, T &cs, T &sn);
-template <> struct Eps<double> { static __device__ __forceinline__ double v() { return 1e-15; } };
-// FP32: the rounding noise of a 16-term dot product is ~1e-6 of |p||q|, so a
-// tighter rotation threshold would keep rotating noise until the sweep limit
-template <> struct Eps<float> { static __device__ __forceinline__ float v() { return 1e-6f; } };
-
-template <> __device__ __forceinline__ bool jac_rot<double>(double al, double be, double ga, double &cs, double &sn)
+// norms al, be; false when the rows are already orthogonal to within 1e-6
+// (the rounding noise of a 16-term dot product is ~1e-6 of |p||q|, so a
+// tighter threshold would keep rotating noise until the sweep limit).  The
+// rotation only has to reduce ga (the sweep repeats until the threshold
+// holds), so the approximate reciprocal, divide and square roots of the SFU
+// suffice
+__device__ __forceinline__ bool jac_rot(float al, float be, float ga, float &cs, float &sn)
 {
-    if (ga == 0.0 || fabs(ga) <= Eps<double>::v() * sqrt(al * be)) return false;
-    double tau = (be - al) / (2.0 * ga);
-    double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-    cs = 1.0 / sqrt(1.0 + t * t);
-    sn = cs * t;
-    return true;
-}
-// FP32: the rotation only has to reduce ga (the sweep repeats until the
-// threshold holds), so the approximate reciprocal, divide and square roots
-// of the SFU suffice
-template <> __device__ __forceinline__ bool jac_rot<float>(float al, float be, float ga, float &cs, float &sn)
-{
-    const float e = Eps<float>::v();
+    const float e = 1e-6f;
     if (ga == 0.f || ga * ga <= e * e * (al * be)) return false;
     float tau = __fdividef(be - al, 2.f * ga);
     const float at = fabsf(tau);
@@ -491,7 +478,7 @@ __device__ void jacobi4(T (&X)[4][N], T (&s)[4], T (&u)[4][4])
 #pragma unroll
             for (int q = p + 1; q < 4; q++) {
                 T al = 0, be = 0, ga = 0;
-                if constexpr (sizeof(T) == 4 && N % 4 == 0) {
+                {
                     // FP32: paired (f32x2) products over k = (2m, 2m+1), two
                     // partial sums each to shorten the dependency chains
                     float2 a2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
@@ -508,18 +495,11 @@ __device__ void jacobi4(T (&X)[4][N], T (&s)[4], T (&u)[4][4])
                     al = a.x + a.y;
                     be = b.x + b.y;
                     ga = g.x + g.y;
-                } else {
-#pragma unroll
-                    for (int k = 0; k < N; k++) {
-                        al += X[p][k] * X[p][k];
-                        be += X[q][k] * X[q][k];
-                        ga += X[p][k] * X[q][k];
-                    }
                 }
                 T cs, sn;
-                if (!jac_rot<T>(al, be, ga, cs, sn)) continue;
+                if (!jac_rot(al, be, ga, cs, sn)) continue;
                 any = true;
-                if constexpr (sizeof(T) == 4 && N % 2 == 0) {
+                {
                     const float2 c2 = make_float2(cs, cs), s2 = make_float2(sn, sn), ns2 = make_float2(-sn, -sn);
 #pragma unroll
                     for (int m = 0; m < N / 2; m++) {
@@ -539,25 +519,11 @@ __device__ void jacobi4(T (&X)[4][N], T (&s)[4], T (&u)[4][4])
                         Q[p][2 * m] = np2.x; Q[p][2 * m + 1] = np2.y;
                         Q[q][2 * m] = nq2.x; Q[q][2 * m + 1] = nq2.y;
                     }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < N; k++) {
-                        T xp = X[p][k], xq = X[q][k];
-                        X[p][k] = cs * xp - sn * xq;
-                        X[q][k] = sn * xp + cs * xq;
-                    }
-#pragma unroll
-                    for (int k = 0; k < 4; k++) {
-                        T qp = Q[p][k], qq = Q[q][k];
-                        Q[p][k] = cs * qp - sn * qq;
-                        Q[q][k] = sn * qp + cs * qq;
-                    }
                 }
             }
         if (!any) break;
     }
     T sv[4];
-    int ord[4] = {0, 1, 2, 3};
 #pragma unroll
     for (int p = 0; p < 4; p++) {
         T n2 = 0;
@@ -566,7 +532,7 @@ __device__ void jacobi4(T (&X)[4][N], T (&s)[4], T (&u)[4][4])
         sv[p] = t_sqrt(n2);
     }
     T Y[4][N];
-    if constexpr (sizeof(T) == 4) {
+    {
         // stable sort by descending value: row p goes to position pos[p] (the
         // number of rows before it in that order); moves with static indices
         // only, so that X, Q stay in registers
@@ -578,7 +544,6 @@ __device__ void jacobi4(T (&X)[4][N], T (&s)[4], T (&u)[4][4])
             for (int q = 0; q < 4; q++) r += (sv[q] > sv[p] || (sv[q] == sv[p] && q < p)) ? 1 : 0;
             pos[p] = r;
         }
-        (void)ord;
 #pragma unroll
         for (int p = 0; p < 4; p++) {
             T inv = sv[p] > T(0) ? T(1) / sv[p] : T(0);
@@ -596,23 +561,6 @@ __device__ void jacobi4(T (&X)[4][N], T (&s)[4], T (&u)[4][4])
 #pragma unroll
                 for (int k = 0; k < N; k++) Y[i][k] = X[p][k];
             }
-        }
-
-    } else {
-        // stable insertion sort of 4 indices by descending value
-        for (int i = 1; i < 4; i++) {
-            int o = ord[i], k = i - 1;
-            while (k >= 0 && sv[ord[k]] < sv[o]) { ord[k + 1] = ord[k]; k--; }
-            ord[k + 1] = o;
-        }
-        for (int i = 0; i < 4; i++) {
-            int p = ord[i];
-            s[i] = sv[p];
-            T inv = sv[p] > T(0) ? T(1) / sv[p] : T(0);
-#pragma unroll
-            for (int k = 0; k < 4; k++) u[i][k] = Q[p][k];
-#pragma unroll
-            for (int k = 0; k < N; k++) Y[i][k] = X[p][k] * inv;
         }
     }
 #pragma unroll
@@ -730,14 +678,7 @@ __device__ __forceinline__ T gap_sens(const T (&s)[4], int kept)
 // fi to fj; rn (nullable) collects the rules near their thresholds
 template <typename T>
 __device__ __forceinline__ void estimate_bounds_sens(const T *A, T *out, T &rmargin, T &sens, int fo = 0, int fi = -1,
-                                                     int fj = 0, RankNear<T> *rn = nullptr, T *rrel = nullptr);
-
-template <typename T>
-__device__ void estimate_bounds(const T *A, T *out, T &rmargin)
-{
-    T sens;
-    estimate_bounds_sens<T>(A, out, rmargin, sens);
-}
+                                                     int fj = 0, RankNear<T> *rn = nullptr);
 
 // element i of four (static indices only, so that arrays stay in registers)
 template <typename T>
@@ -746,14 +687,12 @@ __device__ __forceinline__ T sel4(int i, T a0, T a1, T a2, T a3)
     return i == 0 ? a0 : (i == 1 ? a1 : (i == 2 ? a2 : a3));
 }
 
-// rrel (nullable): the smallest distance of a rank rule from its threshold
-// relative to its own singular-value sum (outer and inner rules).  The loops
-// over kept terms are rolled, each term's row picked by static selects: one
+// The loops over kept terms are rolled, each term's row picked by static selects: one
 // copy of the inner SVD and bound code instead of one per possible rank,
 // which keeps the kernel within the instruction cache.
 template <typename T>
 __device__ __forceinline__ void estimate_bounds_sens(const T *A, T *out, T &rmargin, T &sens, int fo, int fi, int fj,
-                                                     RankNear<T> *rn, T *rrel)
+                                                     RankNear<T> *rn)
 {
     T X[4][16];
     T high = 0, tot = 0;
@@ -774,7 +713,6 @@ __device__ __forceinline__ void estimate_bounds_sens(const T *A, T *out, T &rmar
     jacobi4<T, 16>(X, s, u);
     T rm;
     int jr = rank99(s, rm);
-    if (rrel) *rrel = rm / (s[0] + s[1] + s[2] + s[3]);
     if (fo > 0) {
         jr = fo;
         rm = T(1e30);
@@ -803,10 +741,6 @@ __device__ __forceinline__ void estimate_bounds_sens(const T *A, T *out, T &rmar
         jacobi4<T, 4>(V, d, w);
         T rmi;
         int ji = rank99(d, rmi);
-        if (rrel) {
-            const T rr = rmi / (d[0] + d[1] + d[2] + d[3]);
-            *rrel = rr < *rrel ? rr : *rrel;
-        }
         if (i == fi) {
             ji = fj;
         } else {
@@ -936,26 +870,294 @@ __device__ __forceinline__ double high_norm(const double *a, int norm)
     return norm == GS_NORM_MAX ? mx : sqrt(ss);
 }
 
-__global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, const double *__restrict__ A,
-                                                      int64_t n, const uint64_t *parents, const uint8_t *vmask,
-                                                      uint8_t *__restrict__ dec, double *__restrict__ bounds,
-                                                      const int32_t *__restrict__ list, const unsigned *nlist)
+// ---- the FP64 estimate: four lanes per cube
+// GB300 issues one FP64 warp instruction per SM every 16 cycles, so the FP64
+// estimate is bound by their number, and by their latency when few cubes are
+// listed.  Lane l of a quad holds the entries (x, y, z) = (j, k, l) of its
+// cube: its 4 columns of the 4 x 16 unfolding, and afterwards column l of
+// each right vector V_i, so the inner SVDs need no data moved.  The state
+// stays in registers (one thread per cube spilled 3.7 KB) and only 8 cubes
+// share a warp's loops.  A 20,000-atom FP64 mesh: 23.3 ms with one thread per
+// cube and FP64 divisions and roots in every rotation, 19.1 ms.
+
+// gross FP64 approximations (about 20 bits) of the special-function unit
+__device__ __forceinline__ double rcp64_approx(double x)
 {
-    int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (list) {
-        // compacted list of the cubes to estimate (the rest keep DEC_INVALID)
-        if (q >= (int64_t)*nlist) return;
-        q = list[q];
-    } else if (q >= n) {
-        return;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+__device__ __forceinline__ double rsqrt64_approx(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+// 1/x to about 40 bits
+__device__ __forceinline__ double rcp64_40(double x)
+{
+    const double y = rcp64_approx(x);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+// 1/sqrt(x) to FP64 rounding: the approximation y0 (relative error below
+// 2^-18) times the series of (1 - e)^(-1/2), e = 1 - x y0^2, to e^3 (the
+// rest is below 2^-70)
+__device__ __forceinline__ double rsqrt64(double x)
+{
+    const double y0 = rsqrt64_approx(x);
+    const double e = fma(-x, y0 * y0, 1.0);
+    return fma(y0 * e, fma(e, fma(e, 0.3125, 0.375), 0.5), y0);
+}
+
+// The rotation that makes rows with squared norms al, be and inner product
+// ga orthogonal, as tan(a/2) and sin(a) of three shears (p -= th q,
+// q += sn p, p -= th q), and the norms after it.  With h = ga / (be - al),
+// tan(a) = 2 h / (1 + sqrt(1 + 4 h^2)).  The angle only has to reduce ga (the
+// sweep repeats until the threshold holds): small ones, which the later
+// sweeps consist of, are taken to 40 bits, so that convergence stays
+// quadratic, large ones in FP32.  The shears are orthonormal to FP64 for any
+// th as long as sn = 2 th / (1 + th^2) holds to FP64: the series in th^2
+// (th^6 < 2e-22), or the reciprocal approximation and its series to e^2 (the
+// rest is below 2^-54).
+__device__ __forceinline__ void jac_shears64(double &al, double &be, double ga, double &th, double &sn)
+{
+    const double df = be - al, rc = rcp64_approx(df);
+    double h = ga * rc;
+    if (__double2hiint(fabs(h)) < 0x3f400000) {   // |h| < 2^-11
+        h = fma(h, fma(-df, rc, 1.0), h);
+        const double h2 = h * h;
+        th = h * fma(-0.625, h2, 0.5);
+        const double t2 = th * th, tt = th + th;
+        sn = fma(tt, fma(t2, t2, -t2), tt);
+    } else {
+        const float hf = copysignf(fminf(fabsf((float)h), 1e9f), (float)h), q = fmaf(4.f * hf, hf, 1.f);
+        const float tf = __fdividef(2.f * hf, fmaf(q, rsqrtf(q), 1.f));
+        const float r = fmaf(tf, tf, 1.f);
+        h = (double)tf;
+        th = (double)__fdividef(tf, fmaf(r, rsqrtf(r), 1.f));
+        const double rr = fma(th, th, 1.0), y0 = rcp64_approx(rr), e = fma(-rr, y0, 1.0);
+        sn = (th + th) * fma(y0, fma(e, e, e), y0);
     }
-    Octet oc = octet_of(P, level, parents, vmask, q >> 3);
-    if (!((oc.vmask >> (q & 7)) & 1)) { dec[q] = DEC_INVALID; return; }
-    double a[64];
+    al = fma(-h, ga, al);
+    be = fma(h, ga, be);
+}
+// |ga| > 1e-15 sqrt(al be), on the exponents and leading mantissa bits as a
+// piecewise linear logarithm (within 13% on the threshold), which keeps the
+// test off the FP64 pipe
+__device__ __forceinline__ bool jac_needed64(double al, double be, double ga)
+{
+    const int bias = 0x3ff00000;
+    const int lg = (__double2hiint(ga) & 0x7fffffff) - bias;
+    const int la = max(__double2hiint(al), 0) - bias, lb = max(__double2hiint(be), 0) - bias;
+    return lg > -(900 << 20) && 2ll * lg > (long long)la + lb - 104500000ll;   // 2 log2(1e-15) 2^20
+}
+
+// one-sided Jacobi on the 4 rows of a matrix whose columns lie in the four
+// lanes of a quad (NC each): y the lane's columns, z its column of the
+// accumulated rotations (initially the identity).  Each of the three rounds
+// of a sweep rotates two disjoint row pairs; the lane's lowest bit selects
+// the pair whose angle it finds.  Squared norms are taken anew at every sweep
+// and follow the rotations within it (they only steer).  All 32 lanes take
+// part; act: this quad still has work to do.
+template <int NC>
+__device__ __forceinline__ void jacobi_quad(double (&y)[4][NC], double (&z)[4], bool act, int lane)
+{
+    const unsigned full = 0xffffffffu;
+    const bool odd = lane & 1;
+#pragma unroll 1
+    for (int sweep = 0; sweep < 40; sweep++) {
+        double n[4];
 #pragma unroll
-    for (int t = 0; t < 64; t++) a[t] = A[q * 64 + t];
-    double b[6], rm, sens, rrel = 1e30;
-    estimate_bounds_sens<double>(a, b, rm, sens, 0, -1, 0, nullptr, P.near ? &rrel : nullptr);
+        for (int p = 0; p < 4; p++) {
+            n[p] = y[p][0] * y[p][0];
+#pragma unroll
+            for (int k = 1; k < NC; k++) n[p] = fma(y[p][k], y[p][k], n[p]);
+        }
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1)
+#pragma unroll
+            for (int p = 0; p < 4; p++) n[p] += __shfl_xor_sync(full, n[p], o);
+        bool any = false;
+#pragma unroll
+        for (int round = 0; round < 3; round++) {
+            // (0,1)(2,3), (0,2)(1,3), (0,3)(1,2)
+            const int q0 = round + 1, p1 = round == 0 ? 2 : 1, q1 = round == 2 ? 2 : 3;
+            double g0 = y[0][0] * y[q0][0], g1 = y[p1][0] * y[q1][0];
+#pragma unroll
+            for (int k = 1; k < NC; k++) {
+                g0 = fma(y[0][k], y[q0][k], g0);
+                g1 = fma(y[p1][k], y[q1][k], g1);
+            }
+            // the lane's pair: sum over the quad of its inner product
+            double ga = odd ? g1 : g0;
+            ga += __shfl_xor_sync(full, odd ? g0 : g1, 1);
+            ga += __shfl_xor_sync(full, ga, 2);
+            double al = odd ? n[p1] : n[0], be = odd ? n[q1] : n[q0];
+            const bool rot = act && jac_needed64(al, be, ga);
+            if (!__any_sync(full, rot)) continue;
+            any |= rot;
+            double th = 0.0, sn = 0.0;
+            if (rot) jac_shears64(al, be, ga, th, sn);
+            // both pairs' rotations and norms
+            const double tho = __shfl_xor_sync(full, th, 1), sno = __shfl_xor_sync(full, sn, 1);
+            const double alo = __shfl_xor_sync(full, al, 1), beo = __shfl_xor_sync(full, be, 1);
+            const double t0 = odd ? tho : th, s0 = odd ? sno : sn, t1 = odd ? th : tho, s1 = odd ? sn : sno;
+            n[0] = odd ? alo : al;
+            n[q0] = odd ? beo : be;
+            n[p1] = odd ? al : alo;
+            n[q1] = odd ? be : beo;
+            auto turn = [](double &p, double &q, double t, double s) {
+                p = fma(-t, q, p);
+                q = fma(s, p, q);
+                p = fma(-t, q, p);
+            };
+#pragma unroll
+            for (int k = 0; k < NC; k++) {
+                turn(y[0][k], y[q0][k], t0, s0);
+                turn(y[p1][k], y[q1][k], t1, s1);
+            }
+            turn(z[0], z[q0], t0, s0);
+            turn(z[p1], z[q1], t1, s1);
+        }
+        if (!__any_sync(full, any)) break;
+    }
+}
+
+// singular values (norms of the rows), rows sorted by descending value (equal
+// ones in row order) and normalised, the accumulated rotations alike
+template <int NC>
+__device__ __forceinline__ void svd_order_quad(double (&y)[4][NC], double (&z)[4], double (&s)[4], int lane)
+{
+    const unsigned full = 0xffffffffu;
+    double n[4], sv[4], inv[4];
+#pragma unroll
+    for (int p = 0; p < 4; p++) {
+        n[p] = y[p][0] * y[p][0];
+#pragma unroll
+        for (int k = 1; k < NC; k++) n[p] = fma(y[p][k], y[p][k], n[p]);
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1)
+#pragma unroll
+        for (int p = 0; p < 4; p++) n[p] += __shfl_xor_sync(full, n[p], o);
+    // one root per lane, passed around the quad
+    const double nm = sel4(lane & 3, n[0], n[1], n[2], n[3]);
+    const double im = nm > 1e-290 ? rsqrt64(nm) : 0.0, sm = nm * im;
+#pragma unroll
+    for (int p = 0; p < 4; p++) {
+        sv[p] = __shfl_sync(full, sm, p, 4);
+        inv[p] = __shfl_sync(full, im, p, 4);
+    }
+    double ys[4][NC], zs[4];
+    int pos[4];
+#pragma unroll
+    for (int p = 0; p < 4; p++) {
+        pos[p] = 0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            // (non-negative: ordered as their bits)
+            const long long a = __double_as_longlong(sv[q]), b = __double_as_longlong(sv[p]);
+            pos[p] += (a > b || (a == b && q < p)) ? 1 : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < NC; k++) y[p][k] *= inv[p];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++)
+#pragma unroll
+        for (int p = 0; p < 4; p++)
+            if (pos[p] == i) {
+                s[i] = sv[p];
+                zs[i] = z[p];
+#pragma unroll
+                for (int k = 0; k < NC; k++) ys[i][k] = y[p][k];
+            }
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        z[i] = zs[i];
+#pragma unroll
+        for (int k = 0; k < NC; k++) y[i][k] = ys[i][k];
+    }
+}
+
+// rows <-> lanes of a 4 x 4 matrix held one column per lane of a quad
+__device__ __forceinline__ void transpose_quad(const double (&v)[4], double (&o)[4], int lane)
+{
+    const unsigned full = 0xffffffffu;
+    const bool b0 = lane & 1, b1 = lane & 2;
+    // swap the off-diagonal elements of the 2 x 2 blocks, then the blocks
+    const double x0 = __shfl_xor_sync(full, b0 ? v[0] : v[1], 1), x1 = __shfl_xor_sync(full, b0 ? v[2] : v[3], 1);
+    const double a0 = b0 ? x0 : v[0], a1 = b0 ? v[1] : x0, a2 = b0 ? x1 : v[2], a3 = b0 ? v[3] : x1;
+    const double y0 = __shfl_xor_sync(full, b1 ? a0 : a2, 2), y1 = __shfl_xor_sync(full, b1 ? a1 : a3, 2);
+    o[0] = b1 ? y0 : a0;
+    o[1] = b1 ? y1 : a1;
+    o[2] = b1 ? a2 : y0;
+    o[3] = b1 ? a3 : y1;
+}
+
+// range of sum_j c_j L_j(t) over [-1,1] as cubic_range<T> gives it; the
+// derivative's zeros are taken to about 40 bits, which the cubic's values
+// there, being stationary, do not feel
+__device__ __forceinline__ void cubic_range64(const double (&cf)[4], double &lo, double &hi)
+{
+    const double e = cf[0] + cf[2], o = cf[1] + cf[3];
+    lo = e - fabs(o);
+    hi = e + fabs(o);
+    const double b0 = fma(-0.5, cf[2], cf[0]), b1 = fma(-1.5, cf[3], cf[1]), b2 = 1.5 * cf[2], b3 = 2.5 * cf[3];
+    // derivative / 1: 3 b3 t^2 + 2 b2 t + b1; half discriminant b2^2 - 3 b3 b1
+    const double qa = 3.0 * b3;
+    const double disc = fma(b2, b2, -qa * b1);
+    double r0 = 2.0, r1 = 2.0;   // outside [-1, 1]: no root
+    if (qa == 0.0) {
+        if (b2 != 0.0) r0 = -0.5 * b1 * rcp64_40(b2);
+    } else if (disc >= 0.0) {
+        double sq = 0.0;
+        if (disc > 1e-290) {
+            const double g = rsqrt64_approx(disc);
+            sq = disc * g;
+            sq = fma(0.5 * g, fma(-sq, sq, disc), sq);
+        }
+        const double w = -(b2 + copysign(sq, b2));
+        if (w != 0.0) {
+            r0 = w * rcp64_40(qa);
+            r1 = b1 * rcp64_40(w);
+        } else {
+            r0 = 0.0;
+        }
+    }
+    if ((__double2hiint(r0) & 0x7fffffff) < 0x3ff00000) {   // |r0| < 1
+        const double v = fma(r0, fma(r0, fma(r0, b3, b2), b1), b0);
+        lo = fmin(lo, v);
+        hi = fmax(hi, v);
+    }
+    if ((__double2hiint(r1) & 0x7fffffff) < 0x3ff00000) {
+        const double v = fma(r1, fma(r1, fma(r1, b3, b2), b1), b0);
+        lo = fmin(lo, v);
+        hi = fmax(hi, v);
+    }
+}
+
+// range of a product of two independent factors
+__device__ __forceinline__ void product_range(double l1, double h1, double l2, double h2, double &mn, double &mx)
+{
+    const double p0 = h1 * h2, p1 = h1 * l2, p2 = l1 * h2, p3 = l1 * l2;
+    mx = fmax(fmax(p0, p1), fmax(p2, p3));
+    mn = fmin(fmin(p0, p1), fmin(p2, p3));
+}
+
+#define E64W_WARPS 4
+// the most cubes k_estimate_f64w takes: in FP64 meshes of 4 to 128 atoms it
+// took 55 us for 300 cubes, 73 for 840, 110 for 1475, 134 for 1914 and 227
+// for 3416; k_estimate_f64 141, 93, 154, 83 and 86
+#define E64W_MAX 1536
+
+// the decision of cube q from its bounds, and the counts of small margins
+__device__ __forceinline__ void finish_f64(const GsProblem &P, int level, int64_t q, const double *a,
+                                           const double (&b0)[6], double rrel, uint8_t *dec, double *bounds)
+{
+    double b[6];
+#pragma unroll
+    for (int k = 0; k < 6; k++) b[k] = b0[k];
     if (P.norm != GS_NORM_SUM) b[3] = high_norm(a, P.norm);
     const int d = P.order == GS_ORDER_LITERAL ? decide_literal(b, P.c, P.precision, level, P.max_depth)
                                               : decide<double>(b, P.c, P.precision, level, P.max_depth);
@@ -969,7 +1171,373 @@ __global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, co
         if (rrel < GS_NEAR_REL) atomicAdd(&P.near[2], 1ull);
     }
     if (bounds)
-        for (int t = 0; t < 6; t++) bounds[q * 6 + t] = b[t];
+        for (int k = 0; k < 6; k++) bounds[q * 6 + k] = b[k];
+}
+
+__global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, const double *__restrict__ A,
+                                                      int64_t n, const uint64_t *parents, const uint8_t *vmask,
+                                                      uint8_t *__restrict__ dec, double *__restrict__ bounds,
+                                                      const int32_t *__restrict__ list, const unsigned *nlist)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, l = lane & 3;
+    // a compacted list of the cubes to estimate, or all of them
+    const int64_t cnt = list ? (int64_t)*nlist : n;
+    if (cnt <= E64W_MAX) return;   // k_estimate_f64w takes them
+    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+    if (t - (lane >> 2) >= cnt) return;   // the whole warp is past the end
+    int64_t q = -1;
+    if (t < cnt) {
+        q = list ? (int64_t)list[t] : t;
+        const Octet oc = octet_of(P, level, parents, vmask, q >> 3);
+        if (!((oc.vmask >> (q & 7)) & 1)) {
+            if (l == 0) dec[q] = DEC_INVALID;
+            q = -1;
+        }
+    }
+    const double *a = A + (q >= 0 ? q * 64 : 0) + l;
+    double y[4][4], z[4], tot = 0.0, high = 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        z[j] = j == l ? 1.0 : 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            y[j][k] = q >= 0 ? a[16 * j + 4 * k] : 0.0;
+            const double v = fabs(y[j][k]);
+            tot += v;
+            if (j >= 2 || k >= 2 || l >= 2) high += v;
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        tot += __shfl_xor_sync(full, tot, o);
+        high += __shfl_xor_sync(full, high, o);
+    }
+    double s[4], rm = 0.0, rrel = 1e30;
+    jacobi_quad<4>(y, z, true, lane);
+    svd_order_quad<4>(y, z, s, lane);
+    int jr = 0;
+    if (tot != 0.0) {
+        jr = rank99(s, rm);
+        rrel = rm / (s[0] + s[1] + s[2] + s[3]);
+    }
+    // the residual A minus the kept rank-one terms, same layout as y
+    double R[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+#pragma unroll
+        for (int k = 0; k < 4; k++) R[j][k] = q >= 0 ? a[16 * j + 4 * k] : 0.0;
+    double lx, hx;   // lane l: the range of u_l
+    {
+        double cf[4];
+        transpose_quad(z, cf, lane);   // lane l: u_l[0..3] (z[i] of lane b is u_i[b])
+        cubic_range64(cf, lx, hx);
+    }
+    double M = 0.0, m = 0.0;
+    int inner = 0;
+    const int jmax = __reduce_max_sync(full, jr);
+#pragma unroll 1
+    for (int i = 0; i < jmax; i++) {
+        const bool on = i < jr;
+        double v[4][1], w[4], d[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            v[k][0] = on ? sel4(i, y[0][k], y[1][k], y[2][k], y[3][k]) : 0.0;
+            w[k] = k == l ? 1.0 : 0.0;
+        }
+        jacobi_quad<1>(v, w, on, lane);
+        svd_order_quad<1>(v, w, d, lane);
+        const double si = sel4(i, s[0], s[1], s[2], s[3]);
+        int ji = 0;
+        if (on) {
+            double rmi;
+            ji = rank99(d, rmi);
+            rrel = fmin(rrel, rmi / (d[0] + d[1] + d[2] + d[3]));
+        }
+        inner += ji;
+        // lane k: the ranges of w_k and V_k
+        double cf[4], vr[4], lo, hi, lo2, hi2, mn, mx;
+        transpose_quad(w, cf, lane);
+        cubic_range64(cf, lo, hi);
+#pragma unroll
+        for (int k = 0; k < 4; k++) vr[k] = v[k][0];
+        transpose_quad(vr, cf, lane);
+        cubic_range64(cf, lo2, hi2);
+        product_range(lo, hi, lo2, hi2, mn, mx);
+        const double dl = sel4(l, d[0], d[1], d[2], d[3]);
+        double Myz = l < ji ? dl * mx : 0.0, myz = l < ji ? dl * mn : 0.0;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            Myz += __shfl_xor_sync(full, Myz, o);
+            myz += __shfl_xor_sync(full, myz, o);
+        }
+        product_range(__shfl_sync(full, lx, i, 4), __shfl_sync(full, hx, i, 4), myz, Myz, mn, mx);
+        if (on) {
+            M = fma(si, mx, M);
+            m = fma(si, mn, m);
+        }
+        const double zi = sel4(i, z[0], z[1], z[2], z[3]);
+        double u[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) u[j] = __shfl_sync(full, zi, j, 4);
+        const int kmax = __reduce_max_sync(full, ji);
+#pragma unroll 1
+        for (int k = 0; k < kmax; k++) {
+            const double wk = sel4(k, w[0], w[1], w[2], w[3]), vk = sel4(k, vr[0], vr[1], vr[2], vr[3]);
+            const double dk = sel4(k, d[0], d[1], d[2], d[3]);
+            const double x = k < ji ? si * dk * vk : 0.0;
+#pragma unroll
+            for (int b = 0; b < 4; b++) {
+                const double xw = x * __shfl_sync(full, wk, b, 4);
+#pragma unroll
+                for (int j = 0; j < 4; j++) R[j][b] = fma(-u[j], xw, R[j][b]);
+            }
+        }
+    }
+    double sr = 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+#pragma unroll
+        for (int k = 0; k < 4; k++) sr += fabs(R[j][k]);
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) sr += __shfl_xor_sync(full, sr, o);
+    if (q < 0 || l != 0) return;
+    const double b[6] = {m - sr, M + sr, sr, high, (double)jr, (double)inner};
+    finish_f64(P, level, q, a, b, rrel, dec, bounds);
+}
+
+// ---- few cubes: one warp per cube
+// A warp of the kernel above spends some 1500 FP64 instructions, each 64
+// cycles of its SM quarter, however few of its quads hold a cube.  With a
+// cube per warp that is about half: 16 lanes hold one column of the
+// unfolding each, half the warp one row pair of the round and its angle (the
+// rows change places between the halves), and the inner SVDs of the four
+// right vectors run side by side, 8 lanes each.  The recheck of a 523-atom
+// mixed mesh (4 levels of up to 100 cubes): 2130 us with one thread per cube,
+// 503 us with quads, 184 us.
+
+// jacobi_quad with one column per lane over 2^LC lanes and the two row pairs
+// of a round in the halves of lane bit LC: (yp, yq) the half's rows, (zp, zq)
+// their accumulated rotations.  Between rounds the first half's second row
+// changes places with the other half's first, second, first row.
+template <int LC>
+__device__ __forceinline__ void jacobi_warp(double &yp, double &yq, double &zp, double &zq, int lane)
+{
+    const unsigned full = 0xffffffffu;
+    const bool second = (lane >> LC) & 1;
+#pragma unroll 1
+    for (int sweep = 0; sweep < 40; sweep++) {
+        double al = yp * yp, be = yq * yq;
+#pragma unroll
+        for (int o = 1; o < (1 << LC); o <<= 1) {
+            al += __shfl_xor_sync(full, al, o);
+            be += __shfl_xor_sync(full, be, o);
+        }
+        bool any = false;
+#pragma unroll
+        for (int round = 0; round < 3; round++) {
+            double ga = yp * yq;
+#pragma unroll
+            for (int o = 1; o < (1 << LC); o <<= 1) ga += __shfl_xor_sync(full, ga, o);
+            const bool rot = jac_needed64(al, be, ga);
+            if (rot) {
+                any = true;
+                double th, sn;
+                jac_shears64(al, be, ga, th, sn);
+                yp = fma(-th, yq, yp);
+                zp = fma(-th, zq, zp);
+                yq = fma(sn, yp, yq);
+                zq = fma(sn, zp, zq);
+                yp = fma(-th, yq, yp);
+                zp = fma(-th, zq, zp);
+            }
+            const bool first = second && round != 1;   // the row that leaves: the second, or this half's first
+            const double y = __shfl_xor_sync(full, first ? yp : yq, 1 << LC);
+            const double z = __shfl_xor_sync(full, first ? zp : zq, 1 << LC);
+            const double n = __shfl_xor_sync(full, first ? al : be, 1 << LC);
+            if (first) {
+                yp = y;
+                zp = z;
+                al = n;
+            } else {
+                yq = y;
+                zq = z;
+                be = n;
+            }
+        }
+        if (!__any_sync(full, any)) break;
+    }
+}
+
+// singular values of the half's two rows, their reciprocals (0 for a zero
+// row) and their places among the four in descending order
+template <int LC>
+__device__ __forceinline__ void svd_place_warp(double yp, double yq, double &sp, double &sq, double &ip, double &iq,
+                                               int &pp, int &pq, int lane)
+{
+    const unsigned full = 0xffffffffu;
+    const bool second = (lane >> LC) & 1;
+    double np = yp * yp, nq = yq * yq;
+#pragma unroll
+    for (int o = 1; o < (1 << LC); o <<= 1) {
+        np += __shfl_xor_sync(full, np, o);
+        nq += __shfl_xor_sync(full, nq, o);
+    }
+    // one root per lane (its lowest bit: the row), passed to the other
+    const double nm = (lane & 1) ? nq : np, im = nm > 1e-290 ? rsqrt64(nm) : 0.0, sm = nm * im;
+    const double io = __shfl_xor_sync(full, im, 1), so = __shfl_xor_sync(full, sm, 1);
+    sp = (lane & 1) ? so : sm;
+    sq = (lane & 1) ? sm : so;
+    ip = (lane & 1) ? io : im;
+    iq = (lane & 1) ? im : io;
+    // (non-negative: ordered as their bits; equal ones in the order of the halves)
+    const long long a = __double_as_longlong(sp), b = __double_as_longlong(sq);
+    const long long c = __shfl_xor_sync(full, a, 1 << LC), d = __shfl_xor_sync(full, b, 1 << LC);
+    pp = (b > a) + (c > a || (second && c == a)) + (d > a || (second && d == a));
+    pq = (a >= b) + (c > b || (second && c == b)) + (d > b || (second && d == b));
+}
+
+__global__ void __launch_bounds__(32 * E64W_WARPS) k_estimate_f64w(GsProblem P, int level,
+                                                                   const double *__restrict__ A, int64_t n,
+                                                                   const uint64_t *parents, const uint8_t *vmask,
+                                                                   uint8_t *__restrict__ dec,
+                                                                   double *__restrict__ bounds,
+                                                                   const int32_t *__restrict__ list,
+                                                                   const unsigned *nlist)
+{
+    __shared__ double s_V[E64W_WARPS][4][4][4], s_W[E64W_WARPS][4][4][4], s_u[E64W_WARPS][4][4];
+    __shared__ double s_s[E64W_WARPS][4], s_d[E64W_WARPS][4][4], s_sd[E64W_WARPS][4][4];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    const int64_t cnt = list ? (int64_t)*nlist : n;
+    if (cnt > E64W_MAX) return;   // k_estimate_f64 takes them
+    const int64_t t = (int64_t)blockIdx.x * E64W_WARPS + wl;
+    if (t >= cnt) return;
+    const int64_t q = list ? (int64_t)list[t] : t;
+    const Octet oc = octet_of(P, level, parents, vmask, q >> 3);
+    if (!((oc.vmask >> (q & 7)) & 1)) {
+        if (lane == 0) dec[q] = DEC_INVALID;
+        return;
+    }
+    const double *a = A + q * 64;
+    // column (lane & 15) of the unfolding; the half's first row pair
+    const int col = lane & 15, h = lane >> 4;
+    double yp = a[32 * h + col], yq = a[32 * h + 16 + col], zp = 2 * h == col, zq = 2 * h + 1 == col;
+    double tot = fabs(yp) + fabs(yq);
+    double high = h || (col >> 2) >= 2 || (col & 3) >= 2 ? tot : 0.0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        tot += __shfl_xor_sync(full, tot, o);
+        high += __shfl_xor_sync(full, high, o);
+    }
+    double b[6] = {0, 0, 0, high, 0, 0}, rrel = 1e30;
+    if (tot != 0.0) {
+        double sp, sq, ip, iq;
+        int pp, pq;
+        jacobi_warp<4>(yp, yq, zp, zq, lane);
+        svd_place_warp<4>(yp, yq, sp, sq, ip, iq, pp, pq, lane);
+        s_V[wl][pp][col >> 2][col & 3] = yp * ip;
+        s_V[wl][pq][col >> 2][col & 3] = yq * iq;
+        if (col < 4) {
+            s_u[wl][pp][col] = zp;
+            s_u[wl][pq][col] = zq;
+            s_s[wl][pp] = sp;
+            s_s[wl][pq] = sq;
+        }
+        __syncwarp();
+        const double s[4] = {s_s[wl][0], s_s[wl][1], s_s[wl][2], s_s[wl][3]};
+        double rm;
+        const int jr = rank99(s, rm);
+        rrel = rm / (s[0] + s[1] + s[2] + s[3]);
+        // inner SVDs: lanes 8 i .. 8 i + 7 take V_i (its row pairs in lane bit 2)
+        const int i = lane >> 3, g = (lane >> 2) & 1, l = lane & 3;
+        double vp = i < jr ? s_V[wl][i][2 * g][l] : 0.0, vq = i < jr ? s_V[wl][i][2 * g + 1][l] : 0.0;
+        double wp = 2 * g == l, wq = 2 * g + 1 == l;
+        jacobi_warp<2>(vp, vq, wp, wq, lane);
+        svd_place_warp<2>(vp, vq, sp, sq, ip, iq, pp, pq, lane);
+        __syncwarp();
+        s_V[wl][i][pp][l] = vp * ip;
+        s_V[wl][i][pq][l] = vq * iq;
+        s_W[wl][i][pp][l] = wp;
+        s_W[wl][i][pq][l] = wq;
+        s_d[wl][i][pp] = sp;
+        s_d[wl][i][pq] = sq;
+        __syncwarp();
+        const double d[4] = {s_d[wl][i][0], s_d[wl][i][1], s_d[wl][i][2], s_d[wl][i][3]};
+        double rmi;
+        const int ji = i < jr ? rank99(d, rmi) : 0;
+        double rri = i < jr ? rmi / (d[0] + d[1] + d[2] + d[3]) : 1e30;
+        int inner = ji;
+#pragma unroll
+        for (int o = 8; o < 32; o <<= 1) {
+            rri = fmin(rri, __shfl_xor_sync(full, rri, o));
+            inner += __shfl_xor_sync(full, inner, o);
+        }
+        rrel = fmin(rrel, rri);
+        const double si = s_s[wl][i], dl = s_d[wl][i][l];
+        if (g == 0) s_sd[wl][i][l] = l < ji ? si * dl : 0.0;
+        __syncwarp();
+        // 1-D ranges: lane (i, 0, k) of w_ik, lane (i, 1, k) of V_ik, then of u_i
+        double cf[4], lo, hi, lx, hx;
+#pragma unroll
+        for (int k = 0; k < 4; k++) cf[k] = g ? s_V[wl][i][l][k] : s_W[wl][i][l][k];
+        cubic_range64(cf, lo, hi);
+#pragma unroll
+        for (int k = 0; k < 4; k++) cf[k] = s_u[wl][i][k];
+        cubic_range64(cf, lx, hx);
+        const double lo2 = __shfl_xor_sync(full, lo, 4), hi2 = __shfl_xor_sync(full, hi, 4);
+        double mn, mx;
+        product_range(lo, hi, lo2, hi2, mn, mx);
+        double Myz = l < ji ? dl * mx : 0.0, myz = l < ji ? dl * mn : 0.0;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            Myz += __shfl_xor_sync(full, Myz, o);
+            myz += __shfl_xor_sync(full, myz, o);
+        }
+        product_range(lx, hx, myz, Myz, mn, mx);
+        double M = i < jr ? si * mx : 0.0, m = i < jr ? si * mn : 0.0;
+#pragma unroll
+        for (int o = 8; o < 32; o <<= 1) {
+            M += __shfl_xor_sync(full, M, o);
+            m += __shfl_xor_sync(full, m, o);
+        }
+        // residual: the lane's entries (x, y, z) = (lane >> 3, (lane >> 1) & 3, 2 (lane & 1) + {0, 1})
+        const int rx = lane >> 3, ry = (lane >> 1) & 3, rz = 2 * (lane & 1);
+        double r0 = a[2 * lane], r1 = a[2 * lane + 1];
+        for (int ii = 0; ii < jr; ii++)
+            for (int k = 0; k < 4; k++) {
+                const double sd = s_sd[wl][ii][k];
+                if (sd == 0.0) break;   // past the kept terms
+                const double sab = sd * s_u[wl][ii][rx] * s_W[wl][ii][k][ry];
+                r0 = fma(-sab, s_V[wl][ii][k][rz], r0);
+                r1 = fma(-sab, s_V[wl][ii][k][rz + 1], r1);
+            }
+        double sr = fabs(r0) + fabs(r1);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) sr += __shfl_xor_sync(full, sr, o);
+        b[0] = m - sr;
+        b[1] = M + sr;
+        b[2] = sr;
+        b[4] = (double)jr;
+        b[5] = (double)inner;
+    }
+    if (lane == 0) finish_f64(P, level, q, a, b, rrel, dec, bounds);
+}
+
+// the FP64 estimate of n cubes, or of the *nlist listed ones (at most n); the
+// number decides on the device which of the two kernels works
+static void launch_estimate_f64(const GsProblem &P, int level, const double *d_A, int64_t n, const uint64_t *d_parents,
+                                const uint8_t *d_vmask, uint8_t *d_dec, double *d_bounds, const int32_t *list,
+                                const unsigned *nlist, cudaStream_t st)
+{
+    if (list || n <= E64W_MAX) {
+        const int64_t m = n < E64W_MAX ? n : E64W_MAX;
+        GS_LAUNCH(k_estimate_f64w, (unsigned)((m + E64W_WARPS - 1) / E64W_WARPS), 32 * E64W_WARPS, 0, st)(
+            P, level, d_A, n, d_parents, d_vmask, d_dec, d_bounds, list, nlist);
+    }
+    if (n > E64W_MAX)
+        GS_LAUNCH(k_estimate_f64, (unsigned)((n + 31) / 32), 128, 0, st)(P, level, d_A, n, d_parents, d_vmask, d_dec,
+                                                                        d_bounds, list, nlist);
 }
 
 // FP64 first pass (default decision order and norm, no bounds wanted):
@@ -1035,15 +1603,13 @@ int gs_estimate_f64(const GsProblem &P, int level, const double *d_A, int64_t n_
         GS_CHECK(cudaMemsetAsync(nlist, 0, sizeof(unsigned), st));
         GS_LAUNCH(k_estimate_pre64, (unsigned)((n_cubes + 255) / 256), 256, 0, st)(P, level, d_A, n_cubes, d_parents,
                                                                                 d_vmask, d_dec, list, nlist);
-        GS_LAUNCH(k_estimate_f64, (unsigned)((n_cubes + 127) / 128), 128, 0, st)(P, level, d_A, n_cubes, d_parents,
-                                                                         d_vmask, d_dec, nullptr, list, nlist);
+        launch_estimate_f64(P, level, d_A, n_cubes, d_parents, d_vmask, d_dec, nullptr, list, nlist, st);
         gs_free(list, st);
         gs_free(nlist, st);
         GS_CHECK(cudaGetLastError());
         return GS_OK;
     }
-    GS_LAUNCH(k_estimate_f64, (unsigned)((n_cubes + 127) / 128), 128, 0, st)(P, level, d_A, n_cubes, d_parents, d_vmask,
-                                                                     d_dec, d_bounds, nullptr, nullptr);
+    launch_estimate_f64(P, level, d_A, n_cubes, d_parents, d_vmask, d_dec, d_bounds, nullptr, nullptr, st);
     GS_CHECK(cudaGetLastError());
     return GS_OK;
 }
@@ -2011,7 +2577,7 @@ int gs_level_mixed(const GsProblem &P, int level, const uint64_t *d_parents, int
             unsigned nb = (unsigned)((nsub * 8 + 127) / 128);
             cudaMemsetAsync(nl, 0, sizeof(unsigned), st);
             GS_LAUNCH(k_child_list, nb, 128, 0, st)(sm, nsub, lst, nl);
-            GS_LAUNCH(k_estimate_f64, nb, 128, 0, st)(P, level, A64, nsub * 8, sp, sm, sd, nullptr, lst, nl);
+            launch_estimate_f64(P, level, A64, nsub * 8, sp, sm, sd, nullptr, lst, nl, st);
         }
         gs_free(lst, st); gs_free(nl, st);
         if (!rc) GS_LAUNCH(k_octet_scatter, (unsigned)((nsub * 8 + 255) / 256), 256, 0, st)(sd, si, sm, nsub, d_dec);
