@@ -1228,6 +1228,8 @@ static int group_levels(const std::vector<int64_t> &mols, std::vector<PreMol> &p
     // root grid are masked explicitly, so its root extent is unbounded
     GsProblem P0 = hp[0];
     for (int a = 0; a < 3; a++) P0.nroot[a] = (int64_t)1 << 40;
+    // the 1-D coefficients must hold for the largest cutoff radius of them all
+    for (int g = 1; g < G; g++) P0.pad = std::max(P0.pad, hp[(size_t)g].pad);
     P0.near = d_near;
     uint64_t *parents = nullptr;
     uint8_t *vmask0 = nullptr;
