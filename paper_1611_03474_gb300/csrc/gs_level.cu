@@ -553,8 +553,19 @@ int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const
 }
 
 // ---------------------------------------------------------------- estimation
+// one cube's 64 coefficients (256 B, 16-byte aligned) in 16-byte loads
+__device__ __forceinline__ void load_tensor_f32(const float *__restrict__ src, float *a)
+{
+    const float4 *s4 = reinterpret_cast<const float4 *>(src);
+#pragma unroll
+    for (int t = 0; t < 16; t++) {
+        const float4 v = __ldg(s4 + t);
+        a[4 * t] = v.x; a[4 * t + 1] = v.y; a[4 * t + 2] = v.z; a[4 * t + 3] = v.w;
+    }
+}
+
 // Truncated SVD bounds of section 2.2.2: FP32 one thread per cube, FP64
-// (further down) four lanes per cube.
+// (further down) four lanes or one warp per cube.
 
 template <typename T> __device__ __forceinline__ T t_sqrt(T x);
 template <> __device__ __forceinline__ double t_sqrt<double>(double x) { return sqrt(x); }
@@ -587,13 +598,11 @@ __device__ __forceinline__ bool jac_rot(float al, float be, float ga, float &cs,
 }
 
 // one-sided Jacobi on the 4 rows of X (4 x N): afterwards the rows are
-// orthogonal and X_in = Q^T X_out.  Returns singular values sorted
-// descending in s, with the matching left vectors (rows of Q) in u and the
-// right vectors (normalised rows of X) written back into X in sorted order.
+// orthogonal and X_in = Q^T X_out; sv receives their norms (the singular
+// values, unsorted)
 template <typename T, int N>
-__device__ void jacobi4(T (&X)[4][N], T (&s)[4], T (&u)[4][4])
+__device__ __forceinline__ void jacobi_rows(T (&X)[4][N], T (&Q)[4][4], T (&sv)[4])
 {
-    T Q[4][4];
 #pragma unroll
     for (int a = 0; a < 4; a++)
 #pragma unroll
@@ -650,7 +659,6 @@ __device__ void jacobi4(T (&X)[4][N], T (&s)[4], T (&u)[4][4])
             }
         if (!any) break;
     }
-    T sv[4];
 #pragma unroll
     for (int p = 0; p < 4; p++) {
         T n2 = 0;
@@ -658,74 +666,72 @@ __device__ void jacobi4(T (&X)[4][N], T (&s)[4], T (&u)[4][4])
         for (int k = 0; k < N; k++) n2 += X[p][k] * X[p][k];
         sv[p] = t_sqrt(n2);
     }
-    T Y[4][N];
-    {
-        // stable sort by descending value: row p goes to position pos[p] (the
-        // number of rows before it in that order); moves with static indices
-        // only, so that X, Q stay in registers
-        int pos[4];
-#pragma unroll
-        for (int p = 0; p < 4; p++) {
-            int r = 0;
-#pragma unroll
-            for (int q = 0; q < 4; q++) r += (sv[q] > sv[p] || (sv[q] == sv[p] && q < p)) ? 1 : 0;
-            pos[p] = r;
-        }
-#pragma unroll
-        for (int p = 0; p < 4; p++) {
-            T inv = sv[p] > T(0) ? T(1) / sv[p] : T(0);
-#pragma unroll
-            for (int k = 0; k < N; k++) X[p][k] *= inv;
-        }
-#pragma unroll
-        for (int i = 0; i < 4; i++) {
-#pragma unroll
-            for (int p = 0; p < 4; p++) {
-                if (pos[p] != i) continue;
-                s[i] = sv[p];
-#pragma unroll
-                for (int k = 0; k < 4; k++) u[i][k] = Q[p][k];
-#pragma unroll
-                for (int k = 0; k < N; k++) Y[i][k] = X[p][k];
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int k = 0; k < N; k++) X[i][k] = Y[i][k];
 }
 
-// range of sum_j c_j L_j(t) over [-1,1]
+// the SVD of a 4 x 4 matrix: singular values sorted descending in s, the
+// matching left vectors in u, the right vectors (normalised rows) in X.  The
+// rows are sorted in place by a network of five exchanges.
 template <typename T>
-__device__ __forceinline__ void cubic_range(const T *cf, T &lo, T &hi)
+__device__ __forceinline__ void svd4(T (&X)[4][4], T (&s)[4], T (&u)[4][4])
 {
-    T p1 = cf[0] + cf[1] + cf[2] + cf[3], m1 = cf[0] - cf[1] + cf[2] - cf[3];
-    lo = p1 < m1 ? p1 : m1;
-    hi = p1 < m1 ? m1 : p1;
+    jacobi_rows<T, 4>(X, u, s);
+    auto exchange = [&](int i, int j) {
+        const bool sw = s[j] > s[i];
+        auto sel = [sw](T &p, T &q) {
+            const T a = sw ? q : p, b = sw ? p : q;
+            p = a;
+            q = b;
+        };
+        sel(s[i], s[j]);
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            sel(X[i][k], X[j][k]);
+            sel(u[i][k], u[j][k]);
+        }
+    };
+    exchange(0, 1);
+    exchange(2, 3);
+    exchange(0, 2);
+    exchange(1, 3);
+    exchange(1, 2);
+#pragma unroll
+    for (int p = 0; p < 4; p++) {
+        const T inv = s[p] > T(0) ? T(1) / s[p] : T(0);
+#pragma unroll
+        for (int k = 0; k < 4; k++) X[p][k] *= inv;
+    }
+}
+
+// range of sum_j c_j L_j(t) over [-1,1], FP32; the cubic is stationary at the
+// derivative's zeros, so approximate divisions serve for these
+__device__ __forceinline__ void cubic_range(const float *cf, float &lo, float &hi)
+{
+    const float p1 = cf[0] + cf[1] + cf[2] + cf[3], m1 = cf[0] - cf[1] + cf[2] - cf[3];
+    lo = fminf(p1, m1);
+    hi = fmaxf(p1, m1);
     // derivative 3 b3 t^2 + 2 b2 t + b1 in monomials of the cubic
-    T b0 = cf[0] - T(0.5) * cf[2], b1 = cf[1] - T(1.5) * cf[3], b2 = T(1.5) * cf[2], b3 = T(2.5) * cf[3];
-    T qa = T(3) * b3, qb = T(2) * b2, qc = b1;
-    T r[2];
-    int nr = 0;
-    if (qa == T(0)) {
-        if (qb != T(0)) r[nr++] = -qc / qb;
+    const float b0 = cf[0] - 0.5f * cf[2], b1 = cf[1] - 1.5f * cf[3], b2 = 1.5f * cf[2], b3 = 2.5f * cf[3];
+    const float qa = 3.f * b3, qb = 2.f * b2;
+    float r0 = 2.f, r1 = 2.f;   // outside (-1, 1): no zero
+    if (qa == 0.f) {
+        if (qb != 0.f) r0 = __fdividef(-b1, qb);
     } else {
-        T disc = qb * qb - T(4) * qa * qc;
-        if (disc >= T(0)) {
-            T sq = t_sqrt(disc);
-            T w = qb >= T(0) ? -(qb + sq) / T(2) : -(qb - sq) / T(2);
-            if (w != T(0)) { r[nr++] = w / qa; r[nr++] = qc / w; }
-            else r[nr++] = T(0);
+        const float disc = qb * qb - 4.f * qa * b1;
+        if (disc >= 0.f) {
+            const float w = -0.5f * (qb + copysignf(sqrtf(disc), qb));
+            r0 = w != 0.f ? __fdividef(w, qa) : 0.f;
+            if (w != 0.f) r1 = __fdividef(b1, w);
         }
     }
-    for (int i = 0; i < nr; i++) {
-        T t = r[i];
-        if (t > T(-1) && t < T(1)) {
-            T v = b0 + t * (b1 + t * (b2 + t * b3));
-            lo = v < lo ? v : lo;
-            hi = v > hi ? v : hi;
-        }
+    if (fabsf(r0) < 1.f) {
+        const float v = b0 + r0 * (b1 + r0 * (b2 + r0 * b3));
+        lo = fminf(lo, v);
+        hi = fmaxf(hi, v);
+    }
+    if (fabsf(r1) < 1.f) {
+        const float v = b0 + r1 * (b1 + r1 * (b2 + r1 * b3));
+        lo = fminf(lo, v);
+        hi = fmaxf(hi, v);
     }
 }
 
@@ -803,8 +809,16 @@ __device__ __forceinline__ T gap_sens(const T (&s)[4], int kept)
 
 // fo > 0 forces the outer rank; fi >= 0 forces the inner rank of kept term
 // fi to fj; rn (nullable) collects the rules near their thresholds
+// A: the tensor (global); S: 80 values of shared memory, EST_THREADS apart
+// (the thread's own column), which receive the sorted right and left vectors
+// of the outer SVD.  Kept in registers these took 80 of a thread's 243, and
+// their rows were picked by selects; 8 warps per SM fitted, now 12 (the
+// 1,000,020-atom assembly: 42.6 ms, 32.0 ms).  Four lanes per cube, as in
+// FP64, took 53.4 ms: more instructions per cube than the paired FMAs here.
+#define EST_THREADS 128
+#define EST_SHARED 80
 template <typename T>
-__device__ __forceinline__ void estimate_bounds_sens(const T *A, T *out, T &rmargin, T &sens, int fo = 0, int fi = -1,
+__device__ __forceinline__ void estimate_bounds_sens(const T *A, T *S, T *out, T &rmargin, T &sens, int fo = 0, int fi = -1,
                                                      int fj = 0, RankNear<T> *rn = nullptr);
 
 // element i of four (static indices only, so that arrays stay in registers)
@@ -818,26 +832,43 @@ __device__ __forceinline__ T sel4(int i, T a0, T a1, T a2, T a3)
 // copy of the inner SVD and bound code instead of one per possible rank,
 // which keeps the kernel within the instruction cache.
 template <typename T>
-__device__ __forceinline__ void estimate_bounds_sens(const T *A, T *out, T &rmargin, T &sens, int fo, int fi, int fj,
+__device__ __forceinline__ void estimate_bounds_sens(const T *A, T *S, T *out, T &rmargin, T &sens, int fo, int fi, int fj,
                                                      RankNear<T> *rn)
 {
-    T X[4][16];
+    T s[4];
     T high = 0, tot = 0;
+    {
+        T X[4][16], Q[4][4], sv[4];
+        load_tensor_f32(A, &X[0][0]);
 #pragma unroll
-    for (int j = 0; j < 4; j++)
+        for (int j = 0; j < 4; j++)
 #pragma unroll
-        for (int k = 0; k < 16; k++) {
-            T v = A[16 * j + k];
-            X[j][k] = v;
-            tot += t_abs(v);
-            if (j >= 2 || (k >> 2) >= 2 || (k & 3) >= 2) high += t_abs(v);
+            for (int k = 0; k < 16; k++) {
+                tot += t_abs(X[j][k]);
+                if (j >= 2 || (k >> 2) >= 2 || (k & 3) >= 2) high += t_abs(X[j][k]);
+            }
+        out[3] = high;
+        rmargin = T(1e30);
+        sens = T(0);
+        if (tot == T(0)) { out[0] = out[1] = out[2] = 0; out[4] = 0; out[5] = 0; return; }
+        jacobi_rows<T, 16>(X, Q, sv);
+        // row p goes to its place in descending order (equal values in row order)
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            int pos = 0;
+#pragma unroll
+            for (int q = 0; q < 4; q++) pos += (sv[q] > sv[p] || (sv[q] == sv[p] && q < p)) ? 1 : 0;
+            const T inv = sv[p] > T(0) ? T(1) / sv[p] : T(0);
+            T *row = S + 16 * pos * EST_THREADS, *left = S + (64 + 4 * pos) * EST_THREADS;
+#pragma unroll
+            for (int k = 0; k < 16; k++) row[k * EST_THREADS] = X[p][k] * inv;
+#pragma unroll
+            for (int k = 0; k < 4; k++) left[k * EST_THREADS] = Q[p][k];
+#pragma unroll
+            for (int i = 0; i < 4; i++)
+                if (pos == i) s[i] = sv[p];
         }
-    out[3] = high;
-    rmargin = T(1e30);
-    sens = T(0);
-    if (tot == T(0)) { out[0] = out[1] = out[2] = 0; out[4] = 0; out[5] = 0; return; }
-    T s[4], u[4][4];
-    jacobi4<T, 16>(X, s, u);
+    }
     T rm;
     int jr = rank99(s, rm);
     if (fo > 0) {
@@ -851,21 +882,21 @@ __device__ __forceinline__ void estimate_bounds_sens(const T *A, T *out, T &rmar
     sens = gap_sens<T>(s, jr);
     // R = A minus the kept rank-one terms, subtracted in place
     T R[64];
-#pragma unroll
-    for (int t = 0; t < 64; t++) R[t] = A[t];
+    load_tensor_f32(A, R);
     T M = 0, m = 0;
     int inner = 0;
 #pragma unroll 1
     for (int i = 0; i < jr; i++) {
         T V[4][4], d[4], w[4][4], ui[4];
+        const T *row = S + 16 * i * EST_THREADS, *left = S + (64 + 4 * i) * EST_THREADS;
 #pragma unroll
         for (int k = 0; k < 4; k++)
 #pragma unroll
-            for (int l = 0; l < 4; l++) V[k][l] = sel4(i, X[0][4 * k + l], X[1][4 * k + l], X[2][4 * k + l], X[3][4 * k + l]);
+            for (int l = 0; l < 4; l++) V[k][l] = row[(4 * k + l) * EST_THREADS];
 #pragma unroll
-        for (int a = 0; a < 4; a++) ui[a] = sel4(i, u[0][a], u[1][a], u[2][a], u[3][a]);
+        for (int a = 0; a < 4; a++) ui[a] = left[a * EST_THREADS];
         const T si0 = sel4(i, s[0], s[1], s[2], s[3]);
-        jacobi4<T, 4>(V, d, w);
+        svd4(V, d, w);
         T rmi;
         int ji = rank99(d, rmi);
         if (i == fi) {
@@ -2375,18 +2406,6 @@ int gs_accum_f32(const GsProblem &P, int level, const uint64_t *d_parents, const
 // all terms; together <= 0.36 S.
 #define RANK_FLIP_ALLOW 0.4f
 
-// one cube's 64 coefficients (256 B, 16-byte aligned) in 16-byte loads
-__device__ __forceinline__ void load_tensor_f32(const float *__restrict__ src, float *a)
-{
-    const float4 *s4 = reinterpret_cast<const float4 *>(src);
-#pragma unroll
-    for (int t = 0; t < 16; t++) {
-        const float4 v = __ldg(s4 + t);
-        a[4 * t] = v.x; a[4 * t + 1] = v.y; a[4 * t + 2] = v.z; a[4 * t + 3] = v.w;
-    }
-}
-
-
 // Cubes whose corner values of P~ straddle c by more than the FP32 error of
 // those sums are kept by the FP64 estimate whatever its SVD gives: L <= min P~
 // and max P~ <= U hold for any factorisation, since R = A - A~ is taken
@@ -2448,18 +2467,20 @@ __device__ __forceinline__ bool estimate_fast_f32(const GsProblem &P, int level,
 __device__ __forceinline__ void estimate_full_f32(const GsProblem &P, int level, const float *__restrict__ A,
                                                   const float *__restrict__ E, int64_t q, uint8_t *__restrict__ dec,
                                                   uint8_t *__restrict__ flag, unsigned long long *why_cnt,
-                                                  float *__restrict__ dbg)
+                                                  float *__restrict__ dbg, float *S)
 {
-    float a[64];
-    load_tensor_f32(A + q * 64, a);
     float tot = 0.f;
+    {
+        float a[64];
+        load_tensor_f32(A + q * 64, a);
 #pragma unroll
-    for (int t = 0; t < 64; t++) tot += fabsf(a[t]);
+        for (int t = 0; t < 64; t++) tot += fabsf(a[t]);
+    }
     float b[6], rm;
     float sens;
     RankNear<float> rn;
     rn.m1 = rn.m2 = 1e30f; rn.who = -1; rn.alt = 0; rn.ssum = 0.f;
-    estimate_bounds_sens<float>(a, b, rm, sens, 0, -1, 0, &rn);
+    estimate_bounds_sens<float>(A + q * 64, S, b, rm, sens, 0, -1, 0, &rn);
     const float c = (float)P.c, prec = (float)P.precision;
     int d = decide<float>(b, c, prec, level, P.max_depth);
     float dA = MIXED_KAPPA * E[q] + 1e-7f * tot;
@@ -2530,19 +2551,19 @@ __global__ void __launch_bounds__(256) k_estimate_pre(GsProblem P, int level, co
     if (slow) list[wb + __popc(bal & ((1u << lane) - 1u))] = (int32_t)q;
 }
 
-// MINB: blocks per SM the register allocation is held to (0: none; 3 caps
-// the registers at 168 and spills the rest to local memory), a shape the
-// tuner chooses; the arithmetic is the same
+// MINB: blocks per SM the register allocation is held to (3: 168 registers, 4:
+// 128 with some spilled), a shape the tuner chooses; the arithmetic is the same
 template <int MINB>
-__global__ void __launch_bounds__(128, MINB) k_estimate_f32(GsProblem P, int level, const float *__restrict__ A,
+__global__ void __launch_bounds__(EST_THREADS, MINB) k_estimate_f32(GsProblem P, int level, const float *__restrict__ A,
                                                             const float *__restrict__ E, uint8_t *__restrict__ dec,
                                                             uint8_t *__restrict__ flag, unsigned long long *why_cnt,
                                                             float *__restrict__ dbg, const int32_t *__restrict__ list,
                                                             const unsigned *nlist)
 {
+    __shared__ float s_S[EST_SHARED * EST_THREADS];
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)*nlist) return;
-    estimate_full_f32(P, level, A, E, (int64_t)list[t], dec, flag, why_cnt, dbg);
+    estimate_full_f32(P, level, A, E, (int64_t)list[t], dec, flag, why_cnt, dbg, s_S + threadIdx.x);
 }
 
 // cubes whose FP32 decision rests on one rank rule near its threshold
@@ -2562,24 +2583,24 @@ __global__ void k_alt_list(const uint8_t *flag, int64_t n, int32_t *list, unsign
 // the listed cubes re-estimated under the flipped rank: the decision stands
 // (flag 0) when it is the same with a margin outside the band and no other
 // rule of the flipped estimate is near its threshold; otherwise FP64 decides
-__global__ void __launch_bounds__(128) k_estimate_alt(GsProblem P, int level, const float *__restrict__ A,
+__global__ void __launch_bounds__(EST_THREADS) k_estimate_alt(GsProblem P, int level, const float *__restrict__ A,
                                                       const float *__restrict__ E, const int32_t *__restrict__ list,
                                                       const unsigned *nlist, const uint8_t *__restrict__ dec,
                                                       uint8_t *__restrict__ flag, unsigned long long *why_cnt)
 {
+    __shared__ float s_S[EST_SHARED * EST_THREADS];
     const int64_t nl = (int64_t)*nlist;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nl; t += (int64_t)gridDim.x * blockDim.x) {
     int64_t q = list[t];
     const unsigned code = flag[q];
     const int who = (int)((code >> 3) & 7u) - 1, altr = (int)(code & 7u);
-    float a[64];
     float tot = 0.f;
 #pragma unroll
-    for (int k = 0; k < 64; k++) { a[k] = A[q * 64 + k]; tot += fabsf(a[k]); }
+    for (int k = 0; k < 64; k++) tot += fabsf(A[q * 64 + k]);
     const float c = (float)P.c, prec = (float)P.precision;
     const float dA = MIXED_KAPPA * E[q] + 1e-7f * tot;
     float b2[6], rm2, sens2;
-    estimate_bounds_sens<float>(a, b2, rm2, sens2, who < 0 ? altr : 0, who, who < 0 ? 0 : altr, nullptr);
+    estimate_bounds_sens<float>(A + q * 64, s_S + threadIdx.x, b2, rm2, sens2, who < 0 ? altr : 0, who, who < 0 ? 0 : altr, nullptr);
     const float bAlt = 4.f * (dA + 1e-7f * tot) * (1.f + fminf(sens2, 1e4f));
     const float mc2 = fminf(fabsf(c - b2[0]), fabsf(b2[1] - c));
     const bool ok = rm2 > 32.f * dA + 1e-5f * tot && decide<float>(b2, c, prec, level, P.max_depth) == (int)dec[q] &&
@@ -2610,9 +2631,9 @@ int gs_estimate_f32(const GsProblem &P, int level, const float *d_A, const float
     rc = gs_tune_run("k_estimate_f32", n_cubes, 2, st, [&](int shape, unsigned long long *scratch) {
         unsigned long long *why = scratch ? (d_why ? scratch : nullptr) : d_why;
         if (shape == 0)
-            GS_LAUNCH(k_estimate_f32<0>, grid, 128, 0, st)(P, level, d_A, d_err, d_dec, d_flag, why, d_dbg, list, nlist);
+            GS_LAUNCH(k_estimate_f32<3>, grid, EST_THREADS, 0, st)(P, level, d_A, d_err, d_dec, d_flag, why, d_dbg, list, nlist);
         else
-            GS_LAUNCH(k_estimate_f32<3>, grid, 128, 0, st)(P, level, d_A, d_err, d_dec, d_flag, why, d_dbg, list, nlist);
+            GS_LAUNCH(k_estimate_f32<4>, grid, EST_THREADS, 0, st)(P, level, d_A, d_err, d_dec, d_flag, why, d_dbg, list, nlist);
     });
     gs_free(list, st);
     gs_free(nlist, st);
