@@ -24,6 +24,8 @@
 // without FMA contraction (-fmad=false): geometric predicates (orientation,
 // in-square and branch tests) then round each product and sum once, so
 // exactly degenerate configurations are recognised as such.
+#include <cstring>
+
 #include "gs_host.cuh"
 
 #define TP_MAX 48      // points of a cube whose neighbours across faces and edges have its size
@@ -161,9 +163,24 @@ __device__ __noinline__ int face_arcs(const double *h, double c, int &around00, 
 
 // Where a cube's output goes: triangles are written while fewer than
 // tri_cap have been produced, points only if all of them fit in pt_cap.  The
-// final pass writes at the scanned offsets with unbounded caps; the first
-// pass writes into a fixed per-cube staging slot (caps TRI_STAGE_T,
-// TRI_STAGE_P), so only cubes that overflow it are traced a second time.
+// tracing pass writes into a fixed per-cube staging slot (caps TRI_STAGE_T,
+// TRI_STAGE_P); what does not fit goes to a pool shared by all cubes, at a
+// place reserved when the cube's counts are known: the triangles past the
+// slot's (kept until then as point numbers), and all points of a cube that
+// has too many.  The 10 to 15% of cubes that overflow their slot were traced
+// a second time before: 4.2 ms of a 1,000,020-atom mesh, 4.1 of the 44 ms of
+// an adaptive one, and 0.24 ms of latency in the smallest.  Only when the
+// pool is full is a cube traced again, with unbounded caps at its final
+// offsets.
+struct TriPool {
+    uint64_t *tk, *pk;          // triangle keys [3], point keys
+    double *xyz;                // point coordinates [3]
+    unsigned long long *used;   // triangles reserved << 32 | points reserved
+    unsigned cap;               // room for so many triangles, and so many points
+    uint64_t *off;              // per cube that overflows: its place (as in used), or TRI_AGAIN
+};
+#define TRI_AGAIN 0xFFFFFFFFFFFFFFFFull
+#define TRI_XT 64              // triangles of a cube past the slot's that can wait
 struct TriOut {
     uint64_t *tri_keys;   // [3] per triangle
     uint64_t *pt_keys;
@@ -171,17 +188,54 @@ struct TriOut {
     int64_t tri_off, pt_off;
     int tri_cap, pt_cap;
     int ntri, npt;
+    const TriPool *pool;  // null: no pool
+    unsigned char *xt;    // [TRI_XT][3] with a pool
 };
 #define TRI_STAGE_T 4
 #define TRI_STAGE_P 6
 
-__device__ __forceinline__ void put_tri(TriOut &o, uint64_t a, uint64_t b, uint64_t c)
+__device__ __forceinline__ void put_tri(TriOut &o, const TPt *pts, int a, int b, int c)
 {
     if (o.ntri < o.tri_cap) {
         uint64_t *d = o.tri_keys + 3 * (o.tri_off + o.ntri);
-        d[0] = a; d[1] = b; d[2] = c;
+        d[0] = pts[a].key; d[1] = pts[b].key; d[2] = pts[c].key;
+    } else if (o.pool && o.ntri - o.tri_cap < TRI_XT) {
+        unsigned char *d = o.xt + 3 * (o.ntri - o.tri_cap);
+        d[0] = (unsigned char)a; d[1] = (unsigned char)b; d[2] = (unsigned char)c;
     }
     o.ntri++;
+}
+
+// exclusive prefix sum of v < 128 over the active lanes of mask act, *total
+// their sum
+__device__ __forceinline__ unsigned lanes_prefix(unsigned act, unsigned v, unsigned *total)
+{
+    const unsigned below = (1u << (threadIdx.x & 31)) - 1u;
+    unsigned pre = 0, tot = 0;
+#pragma unroll
+    for (int b = 0; b < 7; b++) {
+        const unsigned m = __ballot_sync(act, (v >> b) & 1u);
+        pre += (unsigned)__popc(m & below) << b;
+        tot += (unsigned)__popc(m) << b;
+    }
+    *total = tot;
+    return pre;
+}
+
+// room for nt triangles and np points of this lane's cube (one addition per
+// warp); false when the pool is full
+__device__ __forceinline__ bool pool_reserve(const TriPool &P, unsigned nt, unsigned np, uint64_t &to, uint64_t &po)
+{
+    const unsigned act = __activemask();
+    unsigned tt, tp;
+    const unsigned et = lanes_prefix(act, nt, &tt), ep = lanes_prefix(act, np, &tp);
+    const int leader = __ffs(act) - 1;
+    unsigned long long base = 0;
+    if ((int)(threadIdx.x & 31) == leader) base = atomicAdd(P.used, (unsigned long long)tt << 32 | tp);
+    base = __shfl_sync(act, base, leader);
+    to = (base >> 32) + et;
+    po = (base & 0xffffffffull) + ep;
+    return to + nt <= P.cap && po + np <= P.cap;
 }
 
 __device__ __forceinline__ double orient(const double *a, const double *b, const double *c, int i, int j)
@@ -273,11 +327,11 @@ __device__ void clip_piece(const TPt *pts, const float (*pf)[3], const unsigned 
         }
         if (pick < 0) { pick = fall; if (degen) atomicAdd(degen, 1ull); }
         int a = v[pick == 0 ? m - 1 : pick - 1], b = v[pick], c = v[pick + 1 == m ? 0 : pick + 1];
-        if (a != b && b != c && a != c) put_tri(o, pts[a].key, pts[b].key, pts[c].key);
+        if (a != b && b != c && a != c) put_tri(o, pts, a, b, c);
         for (int t = pick; t < m - 1; t++) v[t] = v[t + 1];
         m--;
     }
-    if (m == 3 && v[0] != v[1] && v[1] != v[2] && v[0] != v[2]) put_tri(o, pts[v[0]].key, pts[v[1]].key, pts[v[2]].key);
+    if (m == 3 && v[0] != v[1] && v[1] != v[2] && v[0] != v[2]) put_tri(o, pts, v[0], v[1], v[2]);
 }
 
 template <int CAP>
@@ -803,14 +857,36 @@ __device__ int tri_cube(const TriCtx &X, int64_t ci, TriOut &o, unsigned long lo
         if (!ok) return 1;
         if (n >= 3) clip_piece(pts, pf, poly, n, o, degen);
     }
-    // points in world coordinates
-    if (MIX && np <= o.pt_cap) {
-        for (int i = 0; i < np; i++) {
-            double *dst = o.pt_xyz + 3 * (o.pt_off + i);
-            for (int a = 0; a < 3; a++) dst[a] = pw[i][a];
-            o.pt_keys[o.pt_off + i] = pts[i].key;
+    uint64_t *pk = o.pt_keys;
+    double *pxyz = o.pt_xyz;
+    int64_t poff = o.pt_off;
+    bool write = np <= o.pt_cap;
+    if (o.pool && (o.ntri > o.tri_cap || np > o.pt_cap)) {
+        const TriPool &P = *o.pool;
+        const int nx = o.ntri > o.tri_cap ? o.ntri - o.tri_cap : 0;
+        uint64_t to = 0, po = 0;
+        const bool room = pool_reserve(P, nx <= TRI_XT ? (unsigned)nx : 0u, np > o.pt_cap ? (unsigned)np : 0u, to, po);
+        if (room && nx <= TRI_XT) {
+            for (int t = 0; t < 3 * nx; t++) P.tk[3 * to + t] = pts[o.xt[t]].key;
+            if (np > o.pt_cap) {
+                pk = P.pk;
+                pxyz = P.xyz;
+                poff = (int64_t)po;
+                write = true;
+            }
+            P.off[ci] = to << 32 | po;
+        } else {
+            P.off[ci] = TRI_AGAIN;
         }
-    } else if (np <= o.pt_cap) {
+    }
+    // points in world coordinates
+    if (MIX && write) {
+        for (int i = 0; i < np; i++) {
+            double *dst = pxyz + 3 * (poff + i);
+            for (int a = 0; a < 3; a++) dst[a] = pw[i][a];
+            pk[poff + i] = pts[i].key;
+        }
+    } else if (write) {
         double h = ldexp(X.min_edge, X.max_depth - lvl);
         double lo[3], hi[3];
         for (int a = 0; a < 3; a++) {
@@ -818,7 +894,7 @@ __device__ int tri_cube(const TriCtx &X, int64_t ci, TriOut &o, unsigned long lo
             hi[a] = __dadd_rn(X.origin[a], __dmul_rn((double)((C[a] + 1) * sc), X.min_edge));
         }
         for (int i = 0; i < np; i++) {
-            double *dst = o.pt_xyz + 3 * (o.pt_off + i);
+            double *dst = pxyz + 3 * (poff + i);
             for (int a = 0; a < 3; a++) {
                 // the cube's own faces (local 0 or 1, read from the bits)
                 // take the lattice coordinates; lo + (-0) h is lo as well
@@ -828,7 +904,7 @@ __device__ int tri_cube(const TriCtx &X, int64_t ci, TriOut &o, unsigned long lo
                 else if (fb == 0x3FF0000000000000ull) dst[a] = hi[a];
                 else dst[a] = __dadd_rn(lo[a], __dmul_rn(f, h));
             }
-            o.pt_keys[o.pt_off + i] = pts[i].key;
+            pk[poff + i] = pts[i].key;
         }
     }
     o.npt = np;
@@ -1087,10 +1163,11 @@ static int tri_order(const TriCtx &X, int32_t **d_order, int64_t *n_surf, cudaSt
     return GS_OK;
 }
 
-// MIX: over the list of cubes with neighbours of another size (count only);
-// otherwise over all cubes, skipping those
+// MIX: over the list of cubes with neighbours of another size; otherwise over
+// all cubes, skipping those
 template <bool MIX>
-__global__ void __launch_bounds__(128) k_tri_count(TriCtx X, int64_t n_trace, int64_t *__restrict__ ntri,
+__global__ void __launch_bounds__(128) k_tri_count(const __grid_constant__ TriCtx X,
+                                                   const __grid_constant__ TriPool pool, int64_t n_trace, int64_t *__restrict__ ntri,
                                                    int64_t *__restrict__ npt,
                                                    unsigned long long *errs, unsigned long long *surface,
                                                    uint64_t *st_tri, uint64_t *st_pk, double *st_xyz,
@@ -1101,7 +1178,6 @@ __global__ void __launch_bounds__(128) k_tri_count(TriCtx X, int64_t n_trace, in
     if (MIX) {
         if (ci >= (int64_t)*nmlist) return;
         ci = mlist[ci];
-        st_tri = nullptr;
     } else {
         if (ci >= n_trace) return;
         if (order) ci = order[ci];
@@ -1113,6 +1189,9 @@ __global__ void __launch_bounds__(128) k_tri_count(TriCtx X, int64_t n_trace, in
     o.tri_off = ci * TRI_STAGE_T; o.pt_off = ci * TRI_STAGE_P;
     o.tri_cap = st_tri ? TRI_STAGE_T : 0;
     o.pt_cap = st_tri ? TRI_STAGE_P : -1;
+    unsigned char xt[3 * TRI_XT];
+    o.pool = st_tri && pool.tk ? &pool : nullptr;
+    o.xt = xt;
     int bad = tri_cube<MIX>(X, ci, o, st_tri ? degen : nullptr);
     if (bad) { atomicAdd(errs, 1ull); o.ntri = 0; o.npt = 0; }
     {
@@ -1149,27 +1228,33 @@ __device__ __forceinline__ void warp_copy_runs(int len, int excl, int total, int
 }
 
 // staged cubes: copy to the scanned offsets, a warp's 32 cubes together
-// (coalesced stores); the others go to the list of cubes traced again by
-// k_tri_emit
-__global__ void __launch_bounds__(128) k_tri_copy(int64_t n, const int64_t *__restrict__ tri_off,
+// (coalesced stores); a cube that overflowed its slot is copied by the whole
+// warp from the slot and the pool; one that found no room there goes to the
+// list of cubes traced again by k_tri_emit
+__global__ void __launch_bounds__(128) k_tri_copy(int64_t n, const __grid_constant__ TriPool pool,
+                                                  const int64_t *__restrict__ tri_off,
                                                   const int64_t *__restrict__ pt_off, const uint64_t *__restrict__ st_tri,
                                                   const uint64_t *__restrict__ st_pk, const double *__restrict__ st_xyz,
                                                   uint64_t *__restrict__ tri_keys, uint64_t *__restrict__ pt_keys,
                                                   double *__restrict__ pt_xyz, int64_t *__restrict__ redo,
-                                                  unsigned long long *nredo, const uint8_t *__restrict__ mixed)
+                                                  unsigned long long *nredo)
 {
     const unsigned full = 0xffffffffu;
     const int64_t ci = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     bool over = false;
-    int nt = 0, np = 0;
+    int nt = 0, np = 0, ntl = 0, npl = 0;
     int64_t t0 = 0, p0 = 0;
-    if (ci < n && !(mixed && mixed[ci])) {
+    uint64_t place = TRI_AGAIN;
+    if (ci < n) {
         t0 = tri_off[ci];
         p0 = pt_off[ci];
-        const int64_t ntl = tri_off[ci + 1] - t0, npl = pt_off[ci + 1] - p0;
-        if (ntl > TRI_STAGE_T || npl > TRI_STAGE_P) over = true;
-        else { nt = (int)ntl; np = (int)npl; }
+        ntl = (int)(tri_off[ci + 1] - t0);
+        npl = (int)(pt_off[ci + 1] - p0);
+        if (ntl > TRI_STAGE_T || npl > TRI_STAGE_P) {
+            over = true;
+            if (pool.tk) place = pool.off[ci];
+        } else { nt = ntl; np = npl; }
     }
     // runs per lane: 3 nt triangle keys, np point keys, 3 np coordinates
     int it = 3 * nt, ip = np;
@@ -1183,37 +1268,52 @@ __global__ void __launch_bounds__(128) k_tri_copy(int64_t n, const int64_t *__re
     warp_copy_runs<uint64_t>(3 * nt, et, tt, lane, 3 * ci * TRI_STAGE_T, 3 * t0, st_tri, tri_keys);
     warp_copy_runs<uint64_t>(np, ep, tp, lane, ci * TRI_STAGE_P, p0, st_pk, pt_keys);
     warp_copy_runs<double>(3 * np, 3 * ep, 3 * tp, lane, 3 * ci * TRI_STAGE_P, 3 * p0, st_xyz, pt_xyz);
-    const unsigned bal = __ballot_sync(full, over);
+    for (unsigned left = __ballot_sync(full, over && place != TRI_AGAIN); left; left &= left - 1) {
+        const int src = __ffs(left) - 1;
+        const uint64_t pl = __shfl_sync(full, place, src);
+        const int64_t c = __shfl_sync(full, ci, src), td = __shfl_sync(full, t0, src), pd = __shfl_sync(full, p0, src);
+        const int mt = __shfl_sync(full, ntl, src), mp = __shfl_sync(full, npl, src);
+        const uint64_t *pt = pool.tk + 3 * (int64_t)(pl >> 32);
+        for (int k = lane; k < 3 * mt; k += 32)
+            tri_keys[3 * td + k] = k < 3 * TRI_STAGE_T ? st_tri[3 * c * TRI_STAGE_T + k] : pt[k - 3 * TRI_STAGE_T];
+        const int64_t ps = mp > TRI_STAGE_P ? (int64_t)(pl & 0xffffffffull) : c * TRI_STAGE_P;
+        const uint64_t *sk = mp > TRI_STAGE_P ? pool.pk : st_pk;
+        const double *sx = mp > TRI_STAGE_P ? pool.xyz : st_xyz;
+        for (int k = lane; k < mp; k += 32) pt_keys[pd + k] = sk[ps + k];
+        for (int k = lane; k < 3 * mp; k += 32) pt_xyz[3 * pd + k] = sx[3 * ps + k];
+    }
+    const bool again = over && place == TRI_AGAIN;
+    const unsigned bal = __ballot_sync(full, again);
     if (!bal) return;
     unsigned long long base = 0;
     if (lane == 0) base = atomicAdd(nredo, (unsigned long long)__popc(bal));
     base = __shfl_sync(full, base, 0);
-    if (over) redo[base + __popc(bal & ((1u << lane) - 1u))] = ci;
+    if (again) redo[base + __popc(bal & ((1u << lane) - 1u))] = ci;
 }
 
-// final pass over the listed cubes (all cubes when list is null); MIX: the
-// cubes with neighbours of another size, which the other passes skip
+// tracing at the final offsets, over the listed cubes (all cubes when list is
+// null); MIX: the cubes with neighbours of another size, else the others
 template <bool MIX>
-__global__ void __launch_bounds__(128) k_tri_emit(TriCtx X, const int64_t *__restrict__ tri_off,
+__global__ void __launch_bounds__(128) k_tri_emit(const __grid_constant__ TriCtx X,
+                                                  const int64_t *__restrict__ tri_off,
                                                   const int64_t *__restrict__ pt_off, uint64_t *__restrict__ tri_keys,
                                                   uint64_t *__restrict__ pt_keys, double *__restrict__ pt_xyz,
                                                   unsigned long long *degen, const int64_t *__restrict__ list,
                                                   const unsigned long long *nlist)
 {
-    int64_t ci = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (list) {
-        if (ci >= (int64_t)*nlist) return;
-        ci = list[ci];
-    } else if (ci >= X.ncubes) {
-        return;
+    const int64_t n = list ? (int64_t)*nlist : X.ncubes;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t ci = list ? list[t] : t;
+        if ((X.mixed && X.mixed[ci]) != MIX) continue;
+        if (tri_off[ci + 1] == tri_off[ci] && pt_off[ci + 1] == pt_off[ci]) continue;
+        TriOut o;
+        o.ntri = 0; o.npt = 0; o.tri_off = tri_off[ci]; o.pt_off = pt_off[ci];
+        o.tri_cap = 1 << 30; o.pt_cap = 1 << 30;
+        o.tri_keys = tri_keys; o.pt_keys = pt_keys; o.pt_xyz = pt_xyz;
+        o.pool = nullptr;
+        o.xt = nullptr;
+        tri_cube<MIX>(X, ci, o, degen);
     }
-    if (!MIX && X.mixed && X.mixed[ci]) return;
-    if (tri_off[ci + 1] == tri_off[ci] && pt_off[ci + 1] == pt_off[ci]) return;
-    TriOut o;
-    o.ntri = 0; o.npt = 0; o.tri_off = tri_off[ci]; o.pt_off = pt_off[ci];
-    o.tri_cap = 1 << 30; o.pt_cap = 1 << 30;
-    o.tri_keys = tri_keys; o.pt_keys = pt_keys; o.pt_xyz = pt_xyz;
-    tri_cube<MIX>(X, ci, o, degen);
 }
 
 // list of the cubes flagged mixed (any order)
@@ -1248,6 +1348,27 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
         gs_free(st_tri, st); gs_free(st_pk, st); gs_free(st_xyz, st);
         st_tri = nullptr; st_pk = nullptr; st_xyz = nullptr;
     }
+    // and the pool for what the slots do not hold (on average less than one
+    // triangle and one point per cube); without it such cubes are traced twice
+    TriPool pool;
+    memset(&pool, 0, sizeof(pool));
+    if (st_tri && n < ((int64_t)1 << 28)) {   // (the two halves of pool.used stay below 2^32)
+        pool.cap = (unsigned)(n + 4096);
+        if (cudaMallocAsync((void **)&pool.tk, sizeof(uint64_t) * 3 * (size_t)pool.cap, st) != cudaSuccess ||
+            cudaMallocAsync((void **)&pool.pk, sizeof(uint64_t) * (size_t)pool.cap, st) != cudaSuccess ||
+            cudaMallocAsync((void **)&pool.xyz, sizeof(double) * 3 * (size_t)pool.cap, st) != cudaSuccess ||
+            cudaMallocAsync((void **)&pool.off, sizeof(uint64_t) * (size_t)n, st) != cudaSuccess ||
+            cudaMallocAsync((void **)&pool.used, sizeof(unsigned long long), st) != cudaSuccess) {
+            cudaGetLastError();
+            gs_free(pool.tk, st); gs_free(pool.pk, st); gs_free(pool.xyz, st); gs_free(pool.off, st);
+            memset(&pool, 0, sizeof(pool));
+        } else {
+            cudaMemsetAsync(pool.used, 0, sizeof(unsigned long long), st);
+        }
+    }
+    auto free_pool = [&]() {
+        gs_free(pool.tk, st); gs_free(pool.pk, st); gs_free(pool.xyz, st); gs_free(pool.off, st); gs_free(pool.used, st);
+    };
     unsigned nb = (unsigned)((n + 127) / 128);
     // fold-root table; without room for it each cube solves its neighbours' roots
     uint8_t *fcount = nullptr;
@@ -1287,6 +1408,7 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
         gs_free(ntri, st); gs_free(npt, st); gs_free(tot, st);
         gs_free(st_tri, st); gs_free(st_pk, st); gs_free(st_xyz, st);
         gs_free(fcount, st); gs_free(froot, st);
+        free_pool();
         return rc;
     }
     if (order) {
@@ -1295,7 +1417,7 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
     }
     if (n_trace > 0)
         GS_LAUNCH(k_tri_count<false>, (unsigned)((n_trace + 127) / 128), 128, 0, st)(
-            X, n_trace, ntri, npt, d_counters + 0, d_counters + 2, st_tri, st_pk, st_xyz, d_counters + 1, order,
+            X, pool, n_trace, ntri, npt, d_counters + 0, d_counters + 2, st_tri, st_pk, st_xyz, d_counters + 1, order,
             nullptr, nullptr);
     int64_t *mlist = nullptr;
     unsigned long long *nmlist = nullptr;
@@ -1305,8 +1427,8 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
         if (!rc) {
             cudaMemsetAsync(nmlist, 0, sizeof(unsigned long long), st);
             GS_LAUNCH(k_mixed_list, (unsigned)((n + 255) / 256), 256, 0, st)(X.mixed, n, mlist, nmlist);
-            GS_LAUNCH(k_tri_count<true>, nb, 128, 0, st)(X, n, ntri, npt, d_counters + 0, d_counters + 2, nullptr,
-                                                        nullptr, nullptr, d_counters + 1, nullptr, mlist, nmlist);
+            GS_LAUNCH(k_tri_count<true>, nb, 128, 0, st)(X, pool, n, ntri, npt, d_counters + 0, d_counters + 2, st_tri,
+                                                        st_pk, st_xyz, d_counters + 1, nullptr, mlist, nmlist);
         }
     }
     gs_free(order, st);
@@ -1330,19 +1452,25 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
         if (!rc) rc = gs_alloc((void **)&nredo, sizeof(unsigned long long), st);
         if (!rc) {
             cudaMemsetAsync(nredo, 0, sizeof(unsigned long long), st);
-            GS_LAUNCH(k_tri_copy, nb, 128, 0, st)(n, ntri, npt, st_tri, st_pk, st_xyz, *d_tri_keys, *d_pt_keys,
-                                                 *d_pt_xyz, redo, nredo, X.mixed);
-            GS_LAUNCH(k_tri_emit<false>, nb, 128, 0, st)(X, ntri, npt, *d_tri_keys, *d_pt_keys, *d_pt_xyz, nullptr,
+            GS_LAUNCH(k_tri_copy, nb, 128, 0, st)(n, pool, ntri, npt, st_tri, st_pk, st_xyz, *d_tri_keys, *d_pt_keys,
+                                                 *d_pt_xyz, redo, nredo);
+            // normally an empty list
+            const unsigned ne = nb < 152 * 4 ? nb : 152 * 4;
+            GS_LAUNCH(k_tri_emit<false>, ne, 128, 0, st)(X, ntri, npt, *d_tri_keys, *d_pt_keys, *d_pt_xyz, nullptr,
                                                         redo, nredo);
+            if (X.mixed)
+                GS_LAUNCH(k_tri_emit<true>, ne, 128, 0, st)(X, ntri, npt, *d_tri_keys, *d_pt_keys, *d_pt_xyz, nullptr,
+                                                           redo, nredo);
         }
         gs_free(redo, st); gs_free(nredo, st);
     } else if (!rc) {
         GS_LAUNCH(k_tri_emit<false>, nb, 128, 0, st)(X, ntri, npt, *d_tri_keys, *d_pt_keys, *d_pt_xyz, d_counters + 1,
                                                     nullptr, nullptr);
+        if (X.mixed)
+            GS_LAUNCH(k_tri_emit<true>, nb, 128, 0, st)(X, ntri, npt, *d_tri_keys, *d_pt_keys, *d_pt_xyz,
+                                                       d_counters + 1, mlist, nmlist);
     }
-    if (!rc && X.mixed)
-        GS_LAUNCH(k_tri_emit<true>, nb, 128, 0, st)(X, ntri, npt, *d_tri_keys, *d_pt_keys, *d_pt_xyz, d_counters + 1,
-                                                   mlist, nmlist);
+    free_pool();
     gs_free(mlist, st); gs_free(nmlist, st);
     gs_free(st_tri, st); gs_free(st_pk, st); gs_free(st_xyz, st);
     gs_free(fcount, st); gs_free(froot, st);
