@@ -183,19 +183,41 @@ class Mesh:
         self.mismatches = mismatches
 
 
-def _take_host(ptr, n, dtype, shape):
-    if n == 0:
+class _HostArray:
+    """One host array of a library mesh, handed to numpy without a copy: the
+    ndarray made from it (the array interface) keeps it alive, and the memory
+    is released when that array and every view of it are gone.  A copy of
+    the four arrays cost 8.9 of the 51 ms of a 16-molecule batch (98 MB,
+    fresh pages each time)."""
+
+    def __init__(self, mesh, field, shape, typestr, free):
+        kind = type(getattr(mesh, field))
+        addr = ctypes.cast(getattr(mesh, field), ctypes.c_void_p).value
+        self._own = MeshC()
+        setattr(self._own, field, ctypes.cast(addr, kind))
+        setattr(mesh, field, kind())   # the mesh no longer holds it
+        self._free = free
+        self.__array_interface__ = {"data": (addr, False), "shape": shape, "typestr": typestr, "strides": None,
+                                    "version": 3}
+
+    def __del__(self):
+        self._free(ctypes.byref(self._own))
+
+
+def _take_host(mesh, field, shape, dtype, L):
+    dtype = np.dtype(dtype)
+    if int(np.prod(shape)) == 0:
         return np.zeros(shape, dtype=dtype)
-    arr = np.ctypeslib.as_array(ptr, shape=(int(np.prod(shape)),))
-    return np.array(arr, dtype=dtype).reshape(shape)
+    return np.asarray(_HostArray(mesh, field, shape, dtype.str, L.mesh_free))
 
 
 def _mesh_from_c(m, L, stats, max_depth):
     try:
-        res = Mesh(_take_host(m.vertices, m.n_vertices, np.float64, (m.n_vertices, 3)),
-                   _take_host(m.triangles, m.n_triangles, np.int32, (m.n_triangles, 3)),
-                   _take_host(m.vertex_keys, m.n_vertices, np.uint64, (m.n_vertices,)),
-                   _take_host(m.cube_keys, m.n_cubes, np.uint64, (m.n_cubes,)),
+        nv, nt, nc = int(m.n_vertices), int(m.n_triangles), int(m.n_cubes)
+        res = Mesh(_take_host(m, "vertices", (nv, 3), np.float64, L),
+                   _take_host(m, "triangles", (nt, 3), np.int32, L),
+                   _take_host(m, "vertex_keys", (nv,), np.uint64, L),
+                   _take_host(m, "cube_keys", (nc,), np.uint64, L),
                    stats.as_dict(max_depth), m.mismatches)
     finally:
         L.mesh_free(ctypes.byref(m))
