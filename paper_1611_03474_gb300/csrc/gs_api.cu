@@ -369,6 +369,19 @@ static int run_level(const GsProblem &P, int level, const uint64_t *d_parents, i
     auto drop_nexts = [&]() {
         for (size_t i = 0; i < nexts.size(); i++) { gs_free(nexts[i], st); gs_free(nextAs[i], st); gs_free(nextMols[i], st); }
     };
+    struct EventPair {
+        cudaEvent_t e[2] = {nullptr, nullptr};
+        EventPair()
+        {
+            cudaEventCreate(&e[0]);
+            cudaEventCreate(&e[1]);
+        }
+        ~EventPair()
+        {
+            cudaEventDestroy(e[0]);
+            cudaEventDestroy(e[1]);
+        }
+    } acc_ev;
     for (int64_t o0 = 0; o0 < n_oct; o0 += CH) {
         int64_t m = n_oct - o0 < CH ? n_oct - o0 : CH;
         const uint64_t *par = d_parents + o0;
@@ -378,10 +391,9 @@ static int run_level(const GsProblem &P, int level, const uint64_t *d_parents, i
         uint8_t *dec = nullptr;
         int rc = gs_alloc((void **)&dec, (size_t)m * 8, st);
         if (rc) { drop_nexts(); return rc; }
-        float tacc = 0.f;
         if (mode == GS_PREC_MIXED) {
             rc = gs_level_mixed(P, level, par, m, dec, d_pairs, d_rechecked, d_mism, both, d_status, st,
-                                stats ? &tacc : nullptr, d_mism + 1, probs, pmol, pvm);
+                                stats ? acc_ev.e : nullptr, d_mism + 1, probs, pmol, pvm);
         }
         double *dA = nullptr;
         if (mode != GS_PREC_MIXED) {
@@ -389,11 +401,10 @@ static int run_level(const GsProblem &P, int level, const uint64_t *d_parents, i
             if (rc) { gs_free(dec, st); drop_nexts(); return rc; }
             if (reexpand && d_parA) rc = gs_reexpand(d_parA + 64 * o0, m, dA, st);
             else
-                rc = gs_accum_f64(P, level, par, pvm, m, dA, d_pairs, d_status, st, stats ? &tacc : nullptr, probs,
+                rc = gs_accum_f64(P, level, par, pvm, m, dA, d_pairs, d_status, st, stats ? acc_ev.e : nullptr, probs,
                                   pmol);
             if (!rc) rc = gs_estimate_f64(P, level, dA, m * 8, par, pvm, dec, nullptr, st);
         }
-        if (stats) { stats->ms_accum += tacc; stats->n_accum_launches++; }
         if (!rc && lb) rc = gs_level_count_mol(dec, m * 8, pmol, lb->molcnt, st);
         uint64_t *acc = nullptr;
         int32_t *accm = nullptr;
@@ -412,6 +423,13 @@ static int run_level(const GsProblem &P, int level, const uint64_t *d_parents, i
             gs_free(acc, st); gs_free(accm, st); gs_free(nx, st); gs_free(nA, st); gs_free(nm, st);
             drop_nexts();
             return rc;
+        }
+        if (stats) {
+            // the compaction has waited for the stream, so the launch is done
+            float t = 0.f;
+            if (!(reexpand && d_parA)) cudaEventElapsedTime(&t, acc_ev.e[0], acc_ev.e[1]);
+            stats->ms_accum += t;
+            stats->n_accum_launches++;
         }
         acc_parts.push_back(acc);
         acc_counts.push_back(na);

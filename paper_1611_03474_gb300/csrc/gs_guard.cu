@@ -2,8 +2,10 @@
 // for testing the library's error paths without faulting the GPU.
 //
 // gs_sync(st) replaces cudaStreamSynchronize for every host wait of the
-// library: it records an event on the stream and polls it (a short spin,
-// then sleeps of 20 us) until the work is done, a CUDA error comes back, or
+// library: it records an event on the stream and polls it (for 500 us without
+// a pause, then between sleeps of 20 us, which take some 70 us each: more
+// than most waits of a small call) until the work is done, a CUDA error comes
+// back, or
 // the deadline passes (GS_WAIT_TIMEOUT_S seconds, default 600), in which case
 // it returns cudaErrorTimeout and the call returns GS_ERR_TIMEOUT.  Every
 // device loop of the library is bounded, so the deadline only guards
@@ -89,17 +91,15 @@ cudaError_t gs_sync(cudaStream_t st)
     }
     const auto t0 = std::chrono::steady_clock::now();
     const double limit = wait_limit_s();
-    for (long long it = 0;; it++) {
+    for (;;) {
         e = cudaEventQuery(ev);
         if (e != cudaErrorNotReady) break;
-        if (it > 64) {
-            const double dt = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-            if (dt > limit) {
-                e = cudaErrorTimeout;
-                break;
-            }
-            std::this_thread::sleep_for(std::chrono::microseconds(20));
+        const double dt = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+        if (dt > limit) {
+            e = cudaErrorTimeout;
+            break;
         }
+        if (dt > 500e-6) std::this_thread::sleep_for(std::chrono::microseconds(20));
     }
     cudaEventDestroy(ev);
     return e;

@@ -504,13 +504,12 @@ static int grid_for(int64_t n_items, int per_block)
 }
 
 int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const uint8_t *d_vmask, int64_t n_oct,
-                 double *d_A, unsigned long long *d_pairs, unsigned *d_status, cudaStream_t st, float *ms,
+                 double *d_A, unsigned long long *d_pairs, unsigned *d_status, cudaStream_t st, cudaEvent_t *ev,
                  const GsProblem *d_probs, const int32_t *d_mol)
 {
     if (n_oct <= 0) return GS_OK;
     const double hh = 0.5 * gs_h(P, level);
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (ms) { cudaEventCreate(&e0); cudaEventCreate(&e1); cudaEventRecord(e0, st); }
+    if (ev) cudaEventRecord(ev[0], st);
     const unsigned grid = grid_for(n_oct, ACC_WARPS);
     auto run = [&](auto coef) {
         using C = decltype(coef);
@@ -540,14 +539,7 @@ int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const
     }
 #undef GS_ACC64
     (void)d_status;
-    if (ms) {
-        cudaEventRecord(e1, st);
-        cudaEventSynchronize(e1);
-        float t = 0;
-        cudaEventElapsedTime(&t, e0, e1);
-        *ms += t;
-        cudaEventDestroy(e0); cudaEventDestroy(e1);
-    }
+    if (ev) cudaEventRecord(ev[1], st);
     GS_CHECK(cudaGetLastError());
     return GS_OK;
 }
@@ -2316,13 +2308,12 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 4) k_accum_f32(const __grid_co
 }
 
 int gs_accum_f32(const GsProblem &P, int level, const uint64_t *d_parents, const uint8_t *d_vmask, int64_t n_oct,
-                 float *d_A, float *d_err, unsigned long long *d_pairs, unsigned *d_status, cudaStream_t st, float *ms,
+                 float *d_A, float *d_err, unsigned long long *d_pairs, unsigned *d_status, cudaStream_t st, cudaEvent_t *ev,
                  unsigned long long *d_atom_octets, const GsProblem *d_probs, const int32_t *d_mol)
 {
     if (n_oct <= 0) return GS_OK;
     const double h = gs_h(P, level), hh = 0.5 * h;
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (ms) { cudaEventCreate(&e0); cudaEventCreate(&e1); cudaEventRecord(e0, st); }
+    if (ev) cudaEventRecord(ev[0], st);
     // grid shapes the tuner chooses from: up to 64, 16 or 4 blocks per SM
     // (each warp takes every grid-th octet; the sums do not depend on it)
     static const int64_t caps[3] = {152 * 64, 152 * 16, 152 * 4};
@@ -2359,18 +2350,8 @@ int gs_accum_f32(const GsProblem &P, int level, const uint64_t *d_parents, const
         else rc = run("k_accum_f32<nodes16>", Quad32<2, 16>());
     }
 #undef GS_ACC32
-    if (rc) {
-        if (ms) { cudaEventDestroy(e0); cudaEventDestroy(e1); }
-        return rc;
-    }
-    if (ms) {
-        cudaEventRecord(e1, st);
-        cudaEventSynchronize(e1);
-        float t = 0;
-        cudaEventElapsedTime(&t, e0, e1);
-        *ms += t;
-        cudaEventDestroy(e0); cudaEventDestroy(e1);
-    }
+    if (rc) return rc;
+    if (ev) cudaEventRecord(ev[1], st);
     (void)d_status;
     GS_CHECK(cudaGetLastError());
     return GS_OK;
@@ -2743,7 +2724,7 @@ __global__ void k_gather_mol(const int64_t *__restrict__ si, int64_t m, const in
 
 int gs_level_mixed(const GsProblem &P, int level, const uint64_t *d_parents, int64_t n_oct, uint8_t *d_dec,
                    unsigned long long *d_pairs, unsigned long long *d_rechecked, unsigned long long *d_mism,
-                   bool both, unsigned *d_status, cudaStream_t st, float *ms, unsigned long long *d_why,
+                   bool both, unsigned *d_status, cudaStream_t st, cudaEvent_t *ev, unsigned long long *d_why,
                    const GsProblem *d_probs, const int32_t *d_mol, const uint8_t *d_vmask)
 {
     float *A = nullptr, *E = nullptr;
@@ -2755,7 +2736,7 @@ int gs_level_mixed(const GsProblem &P, int level, const uint64_t *d_parents, int
     if (!rc && both) rc = gs_alloc((void **)&dbg, sizeof(float) * 6 * 8 * (size_t)n_oct, st);
     // the counter block holds the atom-octet count 16 slots after the pair count
     if (!rc)
-        rc = gs_accum_f32(P, level, d_parents, d_vmask, n_oct, A, E, d_pairs, d_status, st, ms, d_pairs + 16, d_probs,
+        rc = gs_accum_f32(P, level, d_parents, d_vmask, n_oct, A, E, d_pairs, d_status, st, ev, d_pairs + 16, d_probs,
                           d_mol);
     if (!rc) rc = gs_estimate_f32(P, level, A, E, n_oct * 8, d_parents, d_vmask, d_dec, flag, st, d_why, dbg);
     if (!rc) {

@@ -92,41 +92,71 @@ __device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t *total)
     return before + inc - v;
 }
 
-__global__ void k_scan_tile_sums(const int64_t *__restrict__ v, int64_t n, int64_t *__restrict__ sums)
+// the thread's SCAN_ITEMS consecutive values, in 16-byte loads where all lie
+// in the array and it is aligned for them (8-byte loads touch every sector
+// of the warp's 2 KB twice as often)
+__device__ __forceinline__ bool items_wide(const int64_t *v, int64_t n, int64_t base)
+{
+    return base + SCAN_ITEMS <= n && (reinterpret_cast<uintptr_t>(v) & 15) == 0;
+}
+__device__ __forceinline__ void load_items(const int64_t *__restrict__ v, int64_t n, int64_t base,
+                                           int64_t (&loc)[SCAN_ITEMS])
+{
+    if (items_wide(v, n, base)) {
+        const longlong2 *p = reinterpret_cast<const longlong2 *>(v + base);
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS / 2; i++) {
+            const longlong2 t = p[i];
+            loc[2 * i] = t.x;
+            loc[2 * i + 1] = t.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; i++) loc[i] = base + i < n ? v[base + i] : 0;
+    }
+}
+
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_tile_sums(const int64_t *__restrict__ v, int64_t n,
+                                                                 int64_t *__restrict__ sums)
 {
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-    int64_t s = 0;
+    int64_t loc[SCAN_ITEMS], s = 0;
+    load_items(v, n, base, loc);
 #pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; i++)
-        if (base + i < n) s += v[base + i];
+    for (int i = 0; i < SCAN_ITEMS; i++) s += loc[i];
     int64_t tot;
     block_excl_scan(s, &tot);
     if (threadIdx.x == 0) sums[blockIdx.x] = tot;
 }
 
-__global__ void k_scan_tile_apply(int64_t *__restrict__ v, int64_t n, const int64_t *__restrict__ offs)
+// total (nullable): the sum of all values, from the last thread of the last tile
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_tile_apply(int64_t *__restrict__ v, int64_t n,
+                                                                  const int64_t *__restrict__ offs,
+                                                                  int64_t *__restrict__ total)
 {
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-    int64_t loc[SCAN_ITEMS];
-    int64_t s = 0;
+    int64_t loc[SCAN_ITEMS], s = 0;
+    load_items(v, n, base, loc);
 #pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; i++) {
-        loc[i] = base + i < n ? v[base + i] : 0;
-        s += loc[i];
-    }
+    for (int i = 0; i < SCAN_ITEMS; i++) s += loc[i];
     int64_t tot;
     int64_t pre = block_excl_scan(s, &tot) + (offs ? offs[blockIdx.x] : 0);
+    if (items_wide(v, n, base)) {
+        longlong2 *p = reinterpret_cast<longlong2 *>(v + base);
 #pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; i++) {
-        if (base + i < n) v[base + i] = pre;
-        pre += loc[i];
+        for (int i = 0; i < SCAN_ITEMS / 2; i++) {
+            const int64_t second = pre + loc[2 * i];
+            p[i] = make_longlong2(pre, second);
+            pre = second + loc[2 * i + 1];
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; i++) {
+            if (base + i < n) v[base + i] = pre;
+            pre += loc[i];
+        }
     }
-}
-
-__global__ void k_scan_total(const int64_t *v, const int64_t *orig_last, int64_t n, int64_t *total)
-{
-    // total = exclusive[n-1] + original value at n-1
-    *total = n > 0 ? v[n - 1] + *orig_last : 0;
+    if (total && blockIdx.x == gridDim.x - 1 && threadIdx.x == SCAN_THREADS - 1) *total = pre;
 }
 
 int gs_scan_i64(int64_t *d_vals, int64_t n, int64_t *d_total, cudaStream_t st)
@@ -135,25 +165,19 @@ int gs_scan_i64(int64_t *d_vals, int64_t n, int64_t *d_total, cudaStream_t st)
         if (d_total) GS_CHECK(cudaMemsetAsync(d_total, 0, sizeof(int64_t), st));
         return GS_OK;
     }
-    int64_t *last = nullptr;
-    int rc = gs_alloc((void **)&last, sizeof(int64_t), st);
-    if (rc) return rc;
-    GS_CHECK(cudaMemcpyAsync(last, d_vals + (n - 1), sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
     int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
     if (tiles == 1) {
-        GS_LAUNCH(k_scan_tile_apply, 1, SCAN_THREADS, 0, st)(d_vals, n, nullptr);
+        GS_LAUNCH(k_scan_tile_apply, 1, SCAN_THREADS, 0, st)(d_vals, n, nullptr, d_total);
     } else {
         int64_t *sums = nullptr;
-        rc = gs_alloc((void **)&sums, sizeof(int64_t) * (size_t)tiles, st);
-        if (rc) { gs_free(last, st); return rc; }
+        int rc = gs_alloc((void **)&sums, sizeof(int64_t) * (size_t)tiles, st);
+        if (rc) return rc;
         GS_LAUNCH(k_scan_tile_sums, (unsigned)tiles, SCAN_THREADS, 0, st)(d_vals, n, sums);
         rc = gs_scan_i64(sums, tiles, nullptr, st);
-        if (rc) { gs_free(sums, st); gs_free(last, st); return rc; }
-        GS_LAUNCH(k_scan_tile_apply, (unsigned)tiles, SCAN_THREADS, 0, st)(d_vals, n, sums);
+        if (rc) { gs_free(sums, st); return rc; }
+        GS_LAUNCH(k_scan_tile_apply, (unsigned)tiles, SCAN_THREADS, 0, st)(d_vals, n, sums, d_total);
         gs_free(sums, st);
     }
-    if (d_total) GS_LAUNCH(k_scan_total, 1, 1, 0, st)(d_vals, last, n, d_total);
-    gs_free(last, st);
     GS_CHECK(cudaGetLastError());
     return GS_OK;
 }
