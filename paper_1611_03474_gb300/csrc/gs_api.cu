@@ -821,7 +821,7 @@ static int mesh_impl(const double *atoms, const double *radii, int64_t n, double
     double *phi = nullptr, *raw = nullptr;
     float *err = nullptr, *raw_err = nullptr;
     int64_t *mark = nullptr;
-    GsHash hv{nullptr, nullptr, 0}, hc{nullptr, nullptr, 0};
+    GsHash hv{nullptr, 0}, hc{nullptr, 0};
     uint64_t *vslot = nullptr;
     GsCons K{nullptr, nullptr, nullptr, 0, 0, nullptr, {0}};
     uint8_t *mixed = nullptr;
@@ -842,7 +842,7 @@ static int mesh_impl(const double *atoms, const double *radii, int64_t n, double
         if (!fresh) {
             rc = gs_lattice_vertices(cubes, nc, max_depth, &vkeys, &nv, &cvid, d_status, st, constrain ? &hv : nullptr,
                                      constrain ? &vslot : nullptr);
-            B.keep(vkeys); B.keep(cvid); B.keep(hv.keys); B.keep(hv.vals); B.keep(vslot);
+            B.keep(vkeys); B.keep(cvid); B.keep(hv.kv); B.keep(vslot);
         } else {
             // after splits: the lattice grows by the new cubes' corners
             int64_t added = 0;
@@ -888,7 +888,7 @@ static int mesh_impl(const double *atoms, const double *radii, int64_t n, double
         if (!constrain) break;
         rc = gs_hash_make(&hc, nc, st);
         if (rc) return rc;
-        B.keep(hc.keys); B.keep(hc.vals);
+        B.keep(hc.kv);
         GS_LAUNCH(k_hash_index, (unsigned)((nc + 255) / 256), 256, 0, st)(hc, cubes, nc, d_status);
         rc = gs_cons_alloc(&K, nv, st);
         if (rc) return rc;
@@ -954,9 +954,9 @@ static int mesh_impl(const double *atoms, const double *radii, int64_t n, double
             // this round's lattice grows into the next one's; its raw values
             // and bounds stay with its vertices
             raw_old = raw; err_old = raw_err; nv_keep = nv;
-            release_all({phi, err, mark, hc.keys, hc.vals, K.lev, K.src, K.t, K.list});
+            release_all({phi, err, mark, hc.kv, K.lev, K.src, K.t, K.list});
             phi = nullptr; err = nullptr; mark = nullptr; raw = nullptr; raw_err = nullptr;
-            hc = GsHash{nullptr, nullptr, 0};
+            hc = GsHash{nullptr, 0};
             K = GsCons{nullptr, nullptr, nullptr, 0, 0, nullptr, {0}};
             continue;
         }

@@ -55,7 +55,7 @@ __device__ __forceinline__ int cubes_holding(const GsHash &hc, const int64_t X[3
         const int64_t s = gs_hash_find(hc, gk_make((uint64_t)Q[0], (uint64_t)Q[1], (uint64_t)Q[2], GT_CUBE, (unsigned)l));
         if (s >= 0) {
             found++;
-            if (!f((int64_t)hc.vals[s])) break;
+            if (!f((int64_t)hc.val(s))) break;
         }
     }
     return found;

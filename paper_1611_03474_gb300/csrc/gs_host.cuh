@@ -177,8 +177,8 @@ struct TriCtx {
     // all cubes that share a face or an edge have one size), the cube key ->
     // index table and the lattice-vertex key -> slot table with slot -> id
     const uint8_t *mixed = nullptr;
-    GsHash hc{nullptr, nullptr, 0};
-    GsHash hv{nullptr, nullptr, 0};
+    GsHash hc{nullptr, 0};
+    GsHash hv{nullptr, 0};
     const uint64_t *vslot_id = nullptr;
 };
 // mixed precision: mark (mark[v] = 1) the corners whose FP32 error could move

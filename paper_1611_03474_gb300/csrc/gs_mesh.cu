@@ -17,12 +17,10 @@
 #include <cmath>
 #include <vector>
 
-__global__ void k_hash_clear(uint64_t *keys, uint64_t *vals, uint64_t cap, uint64_t vinit)
+__global__ void k_hash_clear(ulonglong2 *kv, uint64_t cap)
 {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += (uint64_t)gridDim.x * blockDim.x) {
-        keys[i] = GS_EMPTY;
-        if (vals) vals[i] = vinit;
-    }
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += (uint64_t)gridDim.x * blockDim.x)
+        kv[i] = make_ulonglong2(GS_EMPTY, ~0ull);
 }
 
 int gs_hash_make(GsHash *H, int64_t n, cudaStream_t st)
@@ -30,20 +28,19 @@ int gs_hash_make(GsHash *H, int64_t n, cudaStream_t st)
     uint64_t cap = 1024;
     while (cap < (uint64_t)(2 * n + 16)) cap <<= 1;
     H->mask = cap - 1;
-    H->keys = nullptr; H->vals = nullptr;
-    int rc = gs_alloc((void **)&H->keys, sizeof(uint64_t) * cap, st);
-    if (!rc) rc = gs_alloc((void **)&H->vals, sizeof(uint64_t) * cap, st);
-    if (rc) { gs_free(H->keys, st); gs_free(H->vals, st); H->keys = H->vals = nullptr; return rc; }
-    GS_LAUNCH(k_hash_clear, 1024, 256, 0, st)(H->keys, H->vals, cap, ~0ull);
+    H->kv = nullptr;
+    int rc = gs_alloc((void **)&H->kv, sizeof(ulonglong2) * cap, st);
+    if (rc) { H->kv = nullptr; return rc; }
+    const uint64_t nb = (cap + 255) / 256;
+    GS_LAUNCH(k_hash_clear, (unsigned)(nb < 152 * 8 ? nb : 152 * 8), 256, 0, st)(H->kv, cap);
     GS_CHECK(cudaGetLastError());
     return GS_OK;
 }
 
 void gs_hash_free(GsHash *H, cudaStream_t st)
 {
-    gs_free(H->keys, st);
-    gs_free(H->vals, st);
-    H->keys = H->vals = nullptr;
+    gs_free(H->kv, st);
+    H->kv = nullptr;
 }
 
 // insert keys[i] with value i (keys unique)
@@ -52,7 +49,7 @@ __global__ void k_hash_index(GsHash H, const uint64_t *keys, int64_t n, unsigned
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int64_t s = gs_hash_insert(H, keys[i], status);
-    if (s >= 0) H.vals[s] = (uint64_t)i;
+    if (s >= 0) H.set_val(s, (uint64_t)i);
 }
 
 // ---------------------------------------------------------------- conformity
@@ -77,7 +74,7 @@ __global__ void k_conform_mark(GsHash H, const uint64_t *cubes, int64_t n, int64
             int sh = lf - l;
             int64_t s = gs_hash_find(H, gk_make(X >> sh, Y >> sh, Z >> sh, GT_CUBE, (unsigned)l));
             if (s >= 0) {
-                cnt[H.vals[s]] = 8;
+                cnt[H.val(s)] = 8;
                 break;
             }
         }
@@ -210,8 +207,7 @@ __global__ void k_vert_claim(GsHash H, const uint64_t *cubes, int64_t n, int max
     const int leader = __ffs(grp) - 1;
     long long s = -1;
     if (valid && (int)lane == leader) {
-        s = gs_hash_insert(H, key, status);
-        if (s >= 0) atomicMin((unsigned long long *)&H.vals[s], (unsigned long long)t);
+        s = gs_hash_claim(H, key, (uint64_t)t, status);
     }
     s = __shfl_sync(0xffffffffu, s, leader);
     if (valid) slot[t] = (int64_t)s;
@@ -224,7 +220,7 @@ __global__ void k_vert_owner(GsHash H, int64_t n, int64_t *flag, const int64_t *
     if (t >= n * 8) return;
     const int64_t s = slot[t];
     if (s < 0) atomicOr(status, GS_ST_LOOKUP);
-    flag[t] = (s >= 0 && H.vals[s] == (uint64_t)t) ? 1 : 0;
+    flag[t] = (s >= 0 && H.val(s) == (uint64_t)t) ? 1 : 0;
 }
 
 __global__ void k_vert_write(const uint64_t *cubes, int64_t n, int max_depth, const int64_t *off, const int64_t *slot,
@@ -249,7 +245,7 @@ int gs_lattice_vertices(const uint64_t *d_cubes, int64_t n, int max_depth, uint6
                         uint64_t **keep_slot_id)
 {
     *d_vkeys = nullptr; *d_cvid = nullptr; *nv = 0;
-    if (keep_hash) { keep_hash->keys = keep_hash->vals = nullptr; keep_hash->mask = 0; *keep_slot_id = nullptr; }
+    if (keep_hash) { keep_hash->kv = nullptr; keep_hash->mask = 0; *keep_slot_id = nullptr; }
     if (n <= 0) return GS_OK;
     int64_t m = n * 8;
     GsHash H;
@@ -321,9 +317,7 @@ __global__ void k_vert_claim_list(GsHash H, const uint64_t *__restrict__ cubes, 
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= m * 8) return;
     const uint64_t key = corner_key(cubes[list[t >> 3]], (int)(t & 7), max_depth);
-    const int64_t s = gs_hash_insert(H, key, status);
-    if (s >= 0) atomicMin((unsigned long long *)&H.vals[s], (unsigned long long)t);
-    slot[t] = s;
+    slot[t] = gs_hash_claim(H, key, (uint64_t)t, status);
 }
 // a corner owns a new vertex when its slot had no id and it won the slot
 __global__ void k_vert_owner_new(GsHash H, int64_t m, const int64_t *__restrict__ slot,
@@ -333,7 +327,7 @@ __global__ void k_vert_owner_new(GsHash H, int64_t m, const int64_t *__restrict_
     if (t >= m * 8) return;
     const int64_t s = slot[t];
     if (s < 0) atomicOr(status, GS_ST_LOOKUP);
-    flag[t] = (s >= 0 && slot_id[s] == ~0ull && H.vals[s] == (uint64_t)t) ? 1 : 0;
+    flag[t] = (s >= 0 && slot_id[s] == ~0ull && H.val(s) == (uint64_t)t) ? 1 : 0;
 }
 __global__ void k_vert_write_new(const uint64_t *__restrict__ cubes, const int64_t *__restrict__ list, int64_t m,
                                  int max_depth, const int64_t *__restrict__ off, const int64_t *__restrict__ slot,
@@ -436,7 +430,7 @@ __global__ void k_neighbours(GsHash H, const uint64_t *cubes, int64_t n, int32_t
     int32_t r = -1;
     if (c[a] >= 0 && c[a] <= (int64_t)GK_MASK) {
         int64_t s = gs_hash_find(H, gk_make(c[0], c[1], c[2], GT_CUBE, gk_level(k)));
-        if (s >= 0) r = (int32_t)H.vals[s];
+        if (s >= 0) r = (int32_t)H.val(s);
     }
     nbr[t] = r;
 }
@@ -445,7 +439,7 @@ int gs_neighbours(const uint64_t *d_cubes, int64_t n, int32_t **d_nbr, unsigned 
                   GsHash *keep_hash)
 {
     *d_nbr = nullptr;
-    if (keep_hash) { keep_hash->keys = keep_hash->vals = nullptr; keep_hash->mask = 0; }
+    if (keep_hash) { keep_hash->kv = nullptr; keep_hash->mask = 0; }
     if (n <= 0) return GS_OK;
     GsHash H;
     int rc = gs_hash_make(&H, n, st);
@@ -467,16 +461,14 @@ __global__ void k_weld_claim(GsHash H, const uint64_t *pk, int64_t n, int64_t *s
 {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
-    int64_t s = gs_hash_insert(H, pk[t], status);
-    slot[t] = s;
-    if (s >= 0) atomicMin((unsigned long long *)&H.vals[s], (unsigned long long)t);
+    slot[t] = gs_hash_claim(H, pk[t], (uint64_t)t, status);
 }
 __global__ void k_weld_owner(GsHash H, int64_t n, int64_t *flag, const int64_t *slot)
 {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     const int64_t s = slot[t];
-    flag[t] = (s >= 0 && H.vals[s] == (uint64_t)t) ? 1 : 0;
+    flag[t] = (s >= 0 && H.val(s) == (uint64_t)t) ? 1 : 0;
 }
 __global__ void k_weld_write(const uint64_t *pk, const double *pxyz, int64_t n, const int64_t *off, const int64_t *slot,
                              uint64_t *vkeys, double *vxyz, uint64_t *slot_id)

@@ -370,7 +370,7 @@ __device__ __forceinline__ int64_t tri_cube_at(const TriCtx &X, int64_t x, int64
 {
     if (x < 0 || y < 0 || z < 0) return -1;
     const int64_t s = gs_hash_find(X.hc, gk_make((uint64_t)x, (uint64_t)y, (uint64_t)z, GT_CUBE, (unsigned)lvl));
-    return s < 0 ? -1 : (int64_t)X.hc.vals[s];
+    return s < 0 ? -1 : (int64_t)X.hc.val(s);
 }
 // fold roots of axis a of cube q (from the table when there is one)
 __device__ __forceinline__ int cube_fold_roots(const TriCtx &X, int64_t q, int a, double *ru, double *rv)
@@ -1770,7 +1770,7 @@ struct AdjCtx {
 __device__ __forceinline__ int64_t adj_lat(const AdjCtx &C, int64_t x, int64_t y, int64_t z)
 {
     int64_t s = gs_hash_find(C.lat, gk_make(x, y, z, GT_VERT, 0));
-    return s < 0 ? -1 : (int64_t)C.lat.vals[s];
+    return s < 0 ? -1 : (int64_t)C.lat.val(s);
 }
 
 __global__ void __launch_bounds__(128) k_vertex_adjoint(AdjCtx C, unsigned *status)
@@ -1818,7 +1818,7 @@ __global__ void __launch_bounds__(128) k_vertex_adjoint(AdjCtx C, unsigned *stat
     }
     int64_t s = gs_hash_find(C.cub, gk_make(cube[0] / sc, cube[1] / sc, cube[2] / sc, GT_CUBE, lvl));
     if (s < 0) { atomicOr(status, GS_ST_LOOKUP); return; }
-    const int64_t ci = (int64_t)C.cub.vals[s];
+    const int64_t ci = (int64_t)C.cub.val(s);
     double g[8];
     int64_t vid[8];
     for (int v = 0; v < 8; v++) {
