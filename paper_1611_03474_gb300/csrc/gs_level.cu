@@ -325,12 +325,18 @@ struct Series64 {
     }
 };
 
+// split: warps that share an octet, 1 or ACC_WARPS.  With few octets (a recheck)
+// one warp is alone on its SM quarter for an octet's hundreds of atoms: the
+// block's warps then take every fourth 32 candidates each and add their sums
+// at the end (the recheck of 523 atoms, 4 levels: 200 -> 124 us; of 20,000: 510 ->
+// 350).
 // BATCH: octet o belongs to molecule mol[o], whose problem is probs[mol[o]]
 // (the molecules of one launch share D, so one quadrature rule serves all)
 template <class C, bool BATCH>
 __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_constant__ GsProblem P0, int level,
                                                                const uint64_t *parents, const uint8_t *vmask,
-                                                               int64_t n_oct, const __grid_constant__ C coef,
+                                                               int64_t n_oct, int split,
+                                                               const __grid_constant__ C coef,
                                                                double *__restrict__ A_out,
                                                                unsigned long long *pairs,
                                                                const GsProblem *__restrict__ probs,
@@ -342,7 +348,8 @@ __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_const
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1u;
     unsigned long long my_pairs = 0;
-    for (int64_t o = (int64_t)blockIdx.x * ACC_WARPS + wl; o < n_oct; o += (int64_t)gridDim.x * ACC_WARPS) {
+    const int per = ACC_WARPS / split;   // octets of a block
+    for (int64_t o = (int64_t)blockIdx.x * per + wl / split; o < n_oct; o += (int64_t)gridDim.x * per) {
         const GsProblem &P = BATCH ? probs[mol[o]] : P0;
         Octet q = octet_of(P, level, parents, vmask, o);
         int64_t base[3] = {2 * q.I, 2 * q.J, 2 * q.K};
@@ -358,7 +365,7 @@ __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_const
         double acc[16];
 #pragma unroll
         for (int t = 0; t < 16; t++) acc[t] = 0.0;
-        int qn = 0;
+        int qn = 0, part = wl % split;
         const uint8_t vm = q.vmask;
         // update lanes: 4 per (accumulated child, x index); when at most four
         // children are accumulated (a recheck of some cubes of the octet),
@@ -415,6 +422,11 @@ __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_const
         // distance with a margin, the exact FP64 test (the definition) inside
         // the margin
         auto filter = [&](int i) {
+            if (part != 0) {   // another warp's candidates
+                part--;
+                return;
+            }
+            part = split - 1;
             unsigned m = 0;
             if (i >= 0) {
                 const float ah[3] = {P.hx[i], P.hy[i], P.hz[i]}, al[3] = {P.lx[i], P.ly[i], P.lz[i]};
@@ -476,6 +488,20 @@ __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_const
         for (int off = gsz; off < 32; off <<= 1)
 #pragma unroll
             for (int t = 0; t < 16; t++) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], off);
+        if (split > 1) {
+            // the first warp adds the others' sums
+            __syncthreads();
+            if (wl > 0)
+#pragma unroll
+                for (int t = 0; t < 16; t++) s_cf[wl][lane][t] = acc[t];
+            __syncthreads();
+            if (wl == 0)
+                for (int v = 1; v < ACC_WARPS; v++)
+#pragma unroll
+                    for (int t = 0; t < 16; t++) acc[t] += s_cf[v][lane][t];
+            __syncthreads();
+            if (wl > 0) continue;
+        }
         if (pg == 0 && c >= 0) {
             double *dst = A_out + ((size_t)o * 8 + c) * 64 + 16 * j;
 #pragma unroll
@@ -510,14 +536,16 @@ int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const
     if (n_oct <= 0) return GS_OK;
     const double hh = 0.5 * gs_h(P, level);
     if (ev) cudaEventRecord(ev[0], st);
-    const unsigned grid = grid_for(n_oct, ACC_WARPS);
+    // up to four blocks per SM: more octets fill the chip with a warp each
+    const int split = n_oct <= 152 * 4 ? ACC_WARPS : 1;
+    const unsigned grid = grid_for(n_oct, ACC_WARPS / split);
     auto run = [&](auto coef) {
         using C = decltype(coef);
         if (d_probs)
-            GS_LAUNCH((k_accum_f64<C, true>), grid, 32 * ACC_WARPS, 0, st)(P, level, d_parents, d_vmask, n_oct, coef,
+            GS_LAUNCH((k_accum_f64<C, true>), grid, 32 * ACC_WARPS, 0, st)(P, level, d_parents, d_vmask, n_oct, split, coef,
                                                                           d_A, d_pairs, d_probs, d_mol);
         else
-            GS_LAUNCH((k_accum_f64<C, false>), grid, 32 * ACC_WARPS, 0, st)(P, level, d_parents, d_vmask, n_oct, coef,
+            GS_LAUNCH((k_accum_f64<C, false>), grid, 32 * ACC_WARPS, 0, st)(P, level, d_parents, d_vmask, n_oct, split, coef,
                                                                            d_A, d_pairs, nullptr, nullptr);
     };
     // polynomial lengths: a step of one costs 24 of about 330 FP64
