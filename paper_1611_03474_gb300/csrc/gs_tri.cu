@@ -175,9 +175,9 @@ __device__ __noinline__ int face_arcs(const double *h, double c, int &around00, 
 struct TriPool {
     uint64_t *tk, *pk;          // triangle keys [3], point keys
     double *xyz;                // point coordinates [3]
-    unsigned long long *used;   // triangles reserved << 32 | points reserved
+    unsigned long long *used;   // [2] triangles reserved, points reserved
     unsigned cap;               // room for so many triangles, and so many points
-    uint64_t *off;              // per cube that overflows: its place (as in used), or TRI_AGAIN
+    uint64_t *off;              // per cube that overflows: its place (triangle << 32 | point), or TRI_AGAIN
 };
 #define TRI_AGAIN 0xFFFFFFFFFFFFFFFFull
 #define TRI_XT 64              // triangles of a cube past the slot's that can wait
@@ -222,19 +222,22 @@ __device__ __forceinline__ unsigned lanes_prefix(unsigned act, unsigned v, unsig
     return pre;
 }
 
-// room for nt triangles and np points of this lane's cube (one addition per
-// warp); false when the pool is full
+// room for nt triangles and np points of this lane's cube (two additions per
+// warp, in 64 bits: reservations past a full pool count on); false when the
+// pool is full
 __device__ __forceinline__ bool pool_reserve(const TriPool &P, unsigned nt, unsigned np, uint64_t &to, uint64_t &po)
 {
     const unsigned act = __activemask();
     unsigned tt, tp;
     const unsigned et = lanes_prefix(act, nt, &tt), ep = lanes_prefix(act, np, &tp);
     const int leader = __ffs(act) - 1;
-    unsigned long long base = 0;
-    if ((int)(threadIdx.x & 31) == leader) base = atomicAdd(P.used, (unsigned long long)tt << 32 | tp);
-    base = __shfl_sync(act, base, leader);
-    to = (base >> 32) + et;
-    po = (base & 0xffffffffull) + ep;
+    unsigned long long bt = 0, bp = 0;
+    if ((int)(threadIdx.x & 31) == leader) {
+        bt = atomicAdd(P.used, (unsigned long long)tt);
+        bp = atomicAdd(P.used + 1, (unsigned long long)tp);
+    }
+    to = __shfl_sync(act, bt, leader) + et;
+    po = __shfl_sync(act, bp, leader) + ep;
     return to + nt <= P.cap && po + np <= P.cap;
 }
 
@@ -1352,18 +1355,18 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
     // triangle and one point per cube); without it such cubes are traced twice
     TriPool pool;
     memset(&pool, 0, sizeof(pool));
-    if (st_tri && n < ((int64_t)1 << 28)) {   // (the two halves of pool.used stay below 2^32)
+    if (st_tri && n < ((int64_t)1 << 28)) {   // (a place's halves stay below 2^32)
         pool.cap = (unsigned)(n + 4096);
         if (cudaMallocAsync((void **)&pool.tk, sizeof(uint64_t) * 3 * (size_t)pool.cap, st) != cudaSuccess ||
             cudaMallocAsync((void **)&pool.pk, sizeof(uint64_t) * (size_t)pool.cap, st) != cudaSuccess ||
             cudaMallocAsync((void **)&pool.xyz, sizeof(double) * 3 * (size_t)pool.cap, st) != cudaSuccess ||
             cudaMallocAsync((void **)&pool.off, sizeof(uint64_t) * (size_t)n, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&pool.used, sizeof(unsigned long long), st) != cudaSuccess) {
+            cudaMallocAsync((void **)&pool.used, 2 * sizeof(unsigned long long), st) != cudaSuccess) {
             cudaGetLastError();
             gs_free(pool.tk, st); gs_free(pool.pk, st); gs_free(pool.xyz, st); gs_free(pool.off, st);
             memset(&pool, 0, sizeof(pool));
         } else {
-            cudaMemsetAsync(pool.used, 0, sizeof(unsigned long long), st);
+            cudaMemsetAsync(pool.used, 0, 2 * sizeof(unsigned long long), st);
         }
     }
     auto free_pool = [&]() {
