@@ -327,9 +327,11 @@ struct Series64 {
 
 // split: warps that share an octet, 1 or ACC_WARPS.  With few octets (a recheck)
 // one warp is alone on its SM quarter for an octet's hundreds of atoms: the
-// block's warps then take every fourth 32 candidates each and add their sums
-// at the end (the recheck of 523 atoms, 4 levels: 200 -> 124 us; of 20,000: 510 ->
-// 350).
+// block's warps then test every fourth 32 candidates each, compute the
+// coefficients of 128 queued atoms at once and update a quarter of the
+// entries (one k of the four) each.  Atoms are queued in candidate order and
+// every entry adds them in that order in either form, so a cube's tensor
+// does not depend on how many octets share its launch.
 // BATCH: octet o belongs to molecule mol[o], whose problem is probs[mol[o]]
 // (the molecules of one launch share D, so one quadrature rule serves all)
 template <class C, bool BATCH>
@@ -342,11 +344,23 @@ __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_const
                                                                const GsProblem *__restrict__ probs,
                                                                const int32_t *__restrict__ mol)
 {
-    __shared__ double s_cf[ACC_WARPS][32][25];   // per queued atom: 3 axes x 2 intervals x 4 (x times w)
-    __shared__ int s_qi[ACC_WARPS][ACC_Q];
-    __shared__ uint8_t s_qm[ACC_WARPS][ACC_Q];
+    // per queued atom: 3 axes x 2 intervals x 4 (x times w); a warp's part of
+    // these belongs to its octet, or all of them to the block's
+    __shared__ double s_cf[32 * ACC_WARPS][25];
+    __shared__ int s_qi[ACC_Q * ACC_WARPS];
+    __shared__ uint8_t s_qm[ACC_Q * ACC_WARPS];
+    __shared__ int s_n[ACC_WARPS];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const unsigned below = (1u << lane) - 1u;
+    const bool whole = split > 1;   // the block shares an octet
+    const int batch = whole ? 32 * ACC_WARPS : 32, self = whole ? (int)threadIdx.x : lane;
+    double (*cfq)[25] = s_cf + (whole ? 0 : 32 * wl);
+    int *qi = s_qi + (whole ? 0 : ACC_Q * wl);
+    uint8_t *qm = s_qm + (whole ? 0 : ACC_Q * wl);
+    auto sync = [&]() {
+        if (whole) __syncthreads();
+        else __syncwarp();
+    };
     unsigned long long my_pairs = 0;
     const int per = ACC_WARPS / split;   // octets of a block
     for (int64_t o = (int64_t)blockIdx.x * per + wl / split; o < n_oct; o += (int64_t)gridDim.x * per) {
@@ -365,7 +379,8 @@ __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_const
         double acc[16];
 #pragma unroll
         for (int t = 0; t < 16; t++) acc[t] = 0.0;
-        int qn = 0, part = wl % split;
+        int qn = 0, chunk = 0, mine_i = 0;
+        unsigned mine_m = 0;   // whole: the candidate tested for the next merge
         const uint8_t vm = q.vmask;
         // update lanes: 4 per (accumulated child, x index); when at most four
         // children are accumulated (a recheck of some cubes of the octet),
@@ -392,43 +407,79 @@ __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_const
                 need[2] |= 1 << (cc >> 2);
             }
         auto process = [&](int nproc) {
-            if (lane < nproc) {
-                int i = s_qi[wl][lane];
+            if (self < nproc) {
+                int i = qi[self];
                 double xs[3] = {P.ax[i], P.ay[i], P.az[i]};
-                double *cf = s_cf[wl][lane];
+                double *cf = cfq[self];
                 for (int a = 0; a < 3; a++) coef.axis(xs[a], e[a][0], e[a][1], e[a][2], P.D, cf + 8 * a, need[a]);
                 const double w = P.aw[i];
 #pragma unroll
                 for (int k = 0; k < 8; k++)
                     if ((need[0] >> (k >> 2)) & 1) cf[k] *= w;
             }
-            __syncwarp();
-            for (int t = pg; t < nproc; t += G) {
-                if (c >= 0 && ((s_qm[wl][t] >> c) & 1)) {
-                    const double *cf = s_cf[wl][t];
-                    double wa = cf[4 * cx + j];
+            sync();
+            if (whole) {
+                // the warp's entries: k = wl, in acc[0..3]
+                for (int t = pg; t < nproc; t += G) {
+                    if (c >= 0 && ((qm[t] >> c) & 1)) {
+                        const double *cf = cfq[t];
+                        const double wb = cf[4 * cx + j] * cf[8 + 4 * cy + wl];
 #pragma unroll
-                    for (int k = 0; k < 4; k++) {
-                        double wb = wa * cf[8 + 4 * cy + k];
+                        for (int l = 0; l < 4; l++) acc[l] = fma(wb, cf[16 + 4 * cz + l], acc[l]);
+                    }
+                }
+            } else {
+                for (int t = pg; t < nproc; t += G) {
+                    if (c >= 0 && ((qm[t] >> c) & 1)) {
+                        const double *cf = cfq[t];
+                        double wa = cf[4 * cx + j];
 #pragma unroll
-                        for (int l = 0; l < 4; l++) acc[4 * k + l] = fma(wb, cf[16 + 4 * cz + l], acc[4 * k + l]);
+                        for (int k = 0; k < 4; k++) {
+                            double wb = wa * cf[8 + 4 * cy + k];
+#pragma unroll
+                            for (int l = 0; l < 4; l++) acc[4 * k + l] = fma(wb, cf[16 + 4 * cz + l], acc[4 * k + l]);
+                        }
                     }
                 }
             }
-            __syncwarp();
+            sync();
+        };
+        // evaluate the queue's first `batch` members once there are so many
+        auto drain = [&]() {
+            if (qn < batch) return;
+            process(batch);
+            const int rest = qn - batch;
+            int mi = 0;
+            uint8_t mm = 0;
+            if (self < rest) { mi = qi[batch + self]; mm = qm[batch + self]; }
+            sync();
+            if (self < rest) { qi[self] = mi; qm[self] = mm; }
+            sync();
+            qn = rest;
+        };
+        // whole: queue what the warps found in the last ACC_WARPS chunks, in
+        // chunk order (all warps see the same chunks)
+        auto merge = [&]() {
+            const unsigned bal = __ballot_sync(0xffffffffu, mine_m != 0);
+            if (lane == 0) s_n[wl] = __popc(bal);
+            __syncthreads();
+            int pos = qn + __popc(bal & below);
+            for (int v = 0; v < ACC_WARPS; v++) {
+                if (v < wl) pos += s_n[v];
+                qn += s_n[v];
+            }
+            if (mine_m) { qi[pos] = mine_i; qm[pos] = (uint8_t)mine_m; }
+            mine_m = 0;
+            __syncthreads();
+            drain();
         };
 
         // membership of one candidate per lane (i < 0: none): FP32 box
         // distance with a margin, the exact FP64 test (the definition) inside
         // the margin
         auto filter = [&](int i) {
-            if (part != 0) {   // another warp's candidates
-                part--;
-                return;
-            }
-            part = split - 1;
             unsigned m = 0;
-            if (i >= 0) {
+            if (i >= 0 && (!whole || chunk % ACC_WARPS == wl)) {
                 const float ah[3] = {P.hx[i], P.hy[i], P.hz[i]}, al[3] = {P.lx[i], P.ly[i], P.lz[i]};
                 float g2[3][2];
 #pragma unroll
@@ -463,51 +514,39 @@ __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_const
                 }
             }
             my_pairs += __popc(m);
+            if (whole) {
+                if (m) { mine_i = i; mine_m = m; }
+                if (++chunk % ACC_WARPS == 0) merge();
+                return;
+            }
             unsigned bal = __ballot_sync(0xffffffffu, m != 0);
             int pos = qn + __popc(bal & below);
-            if (m) { s_qi[wl][pos] = i; s_qm[wl][pos] = (uint8_t)m; }
+            if (m) { qi[pos] = i; qm[pos] = (uint8_t)m; }
             qn += __popc(bal);
             __syncwarp();
-            if (qn >= 32) {
-                process(32);
-                int rest = qn - 32;
-                int mi = 0; uint8_t mm = 0;
-                if (lane < rest) { mi = s_qi[wl][32 + lane]; mm = s_qm[wl][32 + lane]; }
-                __syncwarp();
-                if (lane < rest) { s_qi[wl][lane] = mi; s_qm[wl][lane] = mm; }
-                __syncwarp();
-                qn = rest;
-            }
+            drain();
         };
 
         if (vm) {
             float flo[3] = {eh[0][0], eh[1][0], eh[2][0]}, fhi[3] = {eh[0][2], eh[1][2], eh[2][2]};
             gs_warp_candidates(P, flo, fhi, lane, filter);
+            if (chunk % ACC_WARPS != 0) merge();
             if (qn > 0) process(qn);
         }
         for (int off = gsz; off < 32; off <<= 1)
 #pragma unroll
             for (int t = 0; t < 16; t++) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], off);
-        if (split > 1) {
-            // the first warp adds the others' sums
-            __syncthreads();
-            if (wl > 0)
-#pragma unroll
-                for (int t = 0; t < 16; t++) s_cf[wl][lane][t] = acc[t];
-            __syncthreads();
-            if (wl == 0)
-                for (int v = 1; v < ACC_WARPS; v++)
-#pragma unroll
-                    for (int t = 0; t < 16; t++) acc[t] += s_cf[v][lane][t];
-            __syncthreads();
-            if (wl > 0) continue;
-        }
         if (pg == 0 && c >= 0) {
             double *dst = A_out + ((size_t)o * 8 + c) * 64 + 16 * j;
+            if (whole) {
 #pragma unroll
-            for (int t = 0; t < 16; t++) dst[t] = acc[t];
+                for (int l = 0; l < 4; l++) dst[4 * wl + l] = acc[l];
+            } else {
+#pragma unroll
+                for (int t = 0; t < 16; t++) dst[t] = acc[t];
+            }
         }
-        if (gsz < 32)   // the children not accumulated hold zeros, as with one lane group
+        if (gsz < 32 && !(whole && wl > 0))   // the children not accumulated hold zeros, as with one lane group
             for (int cc = 0; cc < 8; cc++)
                 if (!((vm >> cc) & 1)) {
                     double *z = A_out + ((size_t)o * 8 + cc) * 64;
