@@ -1229,6 +1229,41 @@ __device__ __forceinline__ bool jac_needed64(double al, double be, double ga)
     return lg > -(900 << 20) && 2ll * lg > (long long)la + lb - 104500000ll;   // 2 log2(1e-15) 2^20
 }
 
+// The two kernels of the FP64 estimate take every sum in the same order and
+// round it alike, so a cube's bounds do not depend on which of them (the
+// length of the list) it meets.  A sum over the 16 columns (k, l) of the
+// unfolding adds fused products over k, then pairs over l; one over all 64
+// entries adds pairs over the rows 2h, 2h + 1, over k, over h and over l.
+// Products and additions that a compiler could contract either way are
+// written as rounded ones.
+
+// the sum over the quad of its lanes' parts
+__device__ __forceinline__ double quad_sum(double v)
+{
+    const unsigned full = 0xffffffffu;
+    v = __dadd_rn(v, __shfl_xor_sync(full, v, 1));
+    return __dadd_rn(v, __shfl_xor_sync(full, v, 2));
+}
+// the lane's part of the inner product of two rows
+template <int NC>
+__device__ __forceinline__ double row_dot(const double (&a)[NC], const double (&b)[NC])
+{
+    double v = __dmul_rn(a[0], b[0]);
+#pragma unroll
+    for (int k = 1; k < NC; k++) v = fma(a[k], b[k], v);
+    return v;
+}
+// the lane's part of a sum over all entries v[j][k]
+__device__ __forceinline__ double entry_sum(const double (&v)[4][4])
+{
+    double t[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+        t[h] = __dadd_rn(__dadd_rn(__dadd_rn(v[2 * h][0], v[2 * h + 1][0]), __dadd_rn(v[2 * h][1], v[2 * h + 1][1])),
+                         __dadd_rn(__dadd_rn(v[2 * h][2], v[2 * h + 1][2]), __dadd_rn(v[2 * h][3], v[2 * h + 1][3])));
+    return __dadd_rn(t[0], t[1]);
+}
+
 // one-sided Jacobi on the 4 rows of a matrix whose columns lie in the four
 // lanes of a quad (NC each): y the lane's columns, z its column of the
 // accumulated rotations (initially the identity).  Each of the three rounds
@@ -1245,30 +1280,16 @@ __device__ __forceinline__ void jacobi_quad(double (&y)[4][NC], double (&z)[4], 
     for (int sweep = 0; sweep < 40; sweep++) {
         double n[4];
 #pragma unroll
-        for (int p = 0; p < 4; p++) {
-            n[p] = y[p][0] * y[p][0];
-#pragma unroll
-            for (int k = 1; k < NC; k++) n[p] = fma(y[p][k], y[p][k], n[p]);
-        }
-#pragma unroll
-        for (int o = 1; o < 4; o <<= 1)
-#pragma unroll
-            for (int p = 0; p < 4; p++) n[p] += __shfl_xor_sync(full, n[p], o);
+        for (int p = 0; p < 4; p++) n[p] = quad_sum(row_dot(y[p], y[p]));
         bool any = false;
 #pragma unroll
         for (int round = 0; round < 3; round++) {
             // (0,1)(2,3), (0,2)(1,3), (0,3)(1,2)
             const int q0 = round + 1, p1 = round == 0 ? 2 : 1, q1 = round == 2 ? 2 : 3;
-            double g0 = y[0][0] * y[q0][0], g1 = y[p1][0] * y[q1][0];
-#pragma unroll
-            for (int k = 1; k < NC; k++) {
-                g0 = fma(y[0][k], y[q0][k], g0);
-                g1 = fma(y[p1][k], y[q1][k], g1);
-            }
+            const double g0 = row_dot(y[0], y[q0]), g1 = row_dot(y[p1], y[q1]);
             // the lane's pair: sum over the quad of its inner product
-            double ga = odd ? g1 : g0;
-            ga += __shfl_xor_sync(full, odd ? g0 : g1, 1);
-            ga += __shfl_xor_sync(full, ga, 2);
+            double ga = __dadd_rn(odd ? g1 : g0, __shfl_xor_sync(full, odd ? g0 : g1, 1));
+            ga = __dadd_rn(ga, __shfl_xor_sync(full, ga, 2));
             double al = odd ? n[p1] : n[0], be = odd ? n[q1] : n[q0];
             const bool rot = act && jac_needed64(al, be, ga);
             if (!__any_sync(full, rot)) continue;
@@ -1308,15 +1329,7 @@ __device__ __forceinline__ void svd_order_quad(double (&y)[4][NC], double (&z)[4
     const unsigned full = 0xffffffffu;
     double n[4], sv[4], inv[4];
 #pragma unroll
-    for (int p = 0; p < 4; p++) {
-        n[p] = y[p][0] * y[p][0];
-#pragma unroll
-        for (int k = 1; k < NC; k++) n[p] = fma(y[p][k], y[p][k], n[p]);
-    }
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1)
-#pragma unroll
-        for (int p = 0; p < 4; p++) n[p] += __shfl_xor_sync(full, n[p], o);
+    for (int p = 0; p < 4; p++) n[p] = quad_sum(row_dot(y[p], y[p]));
     // one root per lane, passed around the quad
     const double nm = sel4(lane & 3, n[0], n[1], n[2], n[3]);
     const double im = nm > 1e-290 ? rsqrt64(nm) : 0.0, sm = nm * im;
@@ -1380,7 +1393,8 @@ __device__ __forceinline__ void cubic_range64(const double (&cf)[4], double &lo,
     const double e = cf[0] + cf[2], o = cf[1] + cf[3];
     lo = e - fabs(o);
     hi = e + fabs(o);
-    const double b0 = fma(-0.5, cf[2], cf[0]), b1 = fma(-1.5, cf[3], cf[1]), b2 = 1.5 * cf[2], b3 = 2.5 * cf[3];
+    const double b0 = fma(-0.5, cf[2], cf[0]), b1 = fma(-1.5, cf[3], cf[1]), b3 = 2.5 * cf[3];
+    const double b2 = fma(1.5, cf[2], 0.0);   // (a zero without its sign, which a rotation by nothing may turn)
     // derivative / 1: 3 b3 t^2 + 2 b2 t + b1; half discriminant b2^2 - 3 b3 b1
     const double qa = 3.0 * b3;
     const double disc = fma(b2, b2, -qa * b1);
@@ -1473,22 +1487,25 @@ __global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, co
         }
     }
     const double *a = A + (q >= 0 ? q * 64 : 0) + l;
-    double y[4][4], z[4], tot = 0.0, high = 0.0;
+    double y[4][4], z[4], tot, high;
+    {
+        double v[4][4];
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-        z[j] = j == l ? 1.0 : 0.0;
+        for (int j = 0; j < 4; j++) {
+            z[j] = j == l ? 1.0 : 0.0;
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
-            y[j][k] = q >= 0 ? a[16 * j + 4 * k] : 0.0;
-            const double v = fabs(y[j][k]);
-            tot += v;
-            if (j >= 2 || k >= 2 || l >= 2) high += v;
+            for (int k = 0; k < 4; k++) {
+                y[j][k] = q >= 0 ? a[16 * j + 4 * k] : 0.0;
+                v[j][k] = fabs(y[j][k]);
+            }
         }
-    }
+        tot = quad_sum(entry_sum(v));
 #pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-        tot += __shfl_xor_sync(full, tot, o);
-        high += __shfl_xor_sync(full, high, o);
+        for (int j = 0; j < 2; j++)
+#pragma unroll
+            for (int k = 0; k < 2; k++)
+                if (l < 2) v[j][k] = 0.0;
+        high = quad_sum(entry_sum(v));
     }
     double s[4], rm = 0.0, rrel = 1e30;
     jacobi_quad<4>(y, z, true, lane);
@@ -1542,12 +1559,8 @@ __global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, co
         cubic_range64(cf, lo2, hi2);
         product_range(lo, hi, lo2, hi2, mn, mx);
         const double dl = sel4(l, d[0], d[1], d[2], d[3]);
-        double Myz = l < ji ? dl * mx : 0.0, myz = l < ji ? dl * mn : 0.0;
-#pragma unroll
-        for (int o = 1; o < 4; o <<= 1) {
-            Myz += __shfl_xor_sync(full, Myz, o);
-            myz += __shfl_xor_sync(full, myz, o);
-        }
+        const double Myz = quad_sum(l < ji ? __dmul_rn(dl, mx) : 0.0);
+        const double myz = quad_sum(l < ji ? __dmul_rn(dl, mn) : 0.0);
         product_range(__shfl_sync(full, lx, i, 4), __shfl_sync(full, hx, i, 4), myz, Myz, mn, mx);
         if (on) {
             M = fma(si, mx, M);
@@ -1571,13 +1584,11 @@ __global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, co
             }
         }
     }
-    double sr = 0.0;
 #pragma unroll
     for (int j = 0; j < 4; j++)
 #pragma unroll
-        for (int k = 0; k < 4; k++) sr += fabs(R[j][k]);
-#pragma unroll
-    for (int o = 1; o < 4; o <<= 1) sr += __shfl_xor_sync(full, sr, o);
+        for (int k = 0; k < 4; k++) R[j][k] = fabs(R[j][k]);
+    const double sr = quad_sum(entry_sum(R));
     if (q < 0 || l != 0) return;
     const double b[6] = {m - sr, M + sr, sr, high, (double)jr, (double)inner};
     finish_f64(P, level, q, a, b, rrel, dec, bounds);
@@ -1593,10 +1604,39 @@ __global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, co
 // mixed mesh (4 levels of up to 100 cubes): 2130 us with one thread per cube,
 // 503 us with quads, 184 us.
 
+// the inner product of two rows with one column per lane, 4 (LC = 2) or 16
+// (LC = 4, column 4 k + l) of them, in the order of row_dot and quad_sum
+template <int LC>
+__device__ __forceinline__ double row_dot_warp(double p, double q, int lane)
+{
+    const unsigned full = 0xffffffffu;
+    double v = __dmul_rn(p, q);
+    if (LC == 4) {
+        const int k = (lane >> 2) & 3;
+#pragma unroll
+        for (int s = 1; s < 4; s++) {
+            const double t = fma(p, q, __shfl_up_sync(full, v, 4));
+            if (k == s) v = t;
+        }
+        v = __shfl_sync(full, v, lane | 12);
+    }
+    return quad_sum(v);
+}
+// the sum over the warp of all entries, lane (h, k, l) holding the sum of
+// those of the rows 2h and 2h + 1, in the order of entry_sum and quad_sum
+__device__ __forceinline__ double entry_sum_warp(double v)
+{
+    const unsigned full = 0xffffffffu;
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) v = __dadd_rn(v, __shfl_xor_sync(full, v, o));
+    return quad_sum(v);
+}
+
 // jacobi_quad with one column per lane over 2^LC lanes and the two row pairs
 // of a round in the halves of lane bit LC: (yp, yq) the half's rows, (zp, zq)
 // their accumulated rotations.  Between rounds the first half's second row
-// changes places with the other half's first, second, first row.
+// changes places with the other half's first, second, first row; after the
+// last round the halves hold the rows 0, 1 and 2, 3 again.
 template <int LC>
 __device__ __forceinline__ void jacobi_warp(double &yp, double &yq, double &zp, double &zq, int lane)
 {
@@ -1604,18 +1644,11 @@ __device__ __forceinline__ void jacobi_warp(double &yp, double &yq, double &zp, 
     const bool second = (lane >> LC) & 1;
 #pragma unroll 1
     for (int sweep = 0; sweep < 40; sweep++) {
-        double al = yp * yp, be = yq * yq;
-#pragma unroll
-        for (int o = 1; o < (1 << LC); o <<= 1) {
-            al += __shfl_xor_sync(full, al, o);
-            be += __shfl_xor_sync(full, be, o);
-        }
+        double al = row_dot_warp<LC>(yp, yp, lane), be = row_dot_warp<LC>(yq, yq, lane);
         bool any = false;
 #pragma unroll
         for (int round = 0; round < 3; round++) {
-            double ga = yp * yq;
-#pragma unroll
-            for (int o = 1; o < (1 << LC); o <<= 1) ga += __shfl_xor_sync(full, ga, o);
+            const double ga = row_dot_warp<LC>(yp, yq, lane);
             const bool rot = jac_needed64(al, be, ga);
             if (rot) {
                 any = true;
@@ -1632,7 +1665,14 @@ __device__ __forceinline__ void jacobi_warp(double &yp, double &yq, double &zp, 
             const double y = __shfl_xor_sync(full, first ? yp : yq, 1 << LC);
             const double z = __shfl_xor_sync(full, first ? zp : zq, 1 << LC);
             const double n = __shfl_xor_sync(full, first ? al : be, 1 << LC);
-            if (first) {
+            if (first && round == 2) {
+                yp = yq;
+                zp = zq;
+                al = be;
+                yq = y;
+                zq = z;
+                be = n;
+            } else if (first) {
                 yp = y;
                 zp = z;
                 al = n;
@@ -1654,12 +1694,7 @@ __device__ __forceinline__ void svd_place_warp(double yp, double yq, double &sp,
 {
     const unsigned full = 0xffffffffu;
     const bool second = (lane >> LC) & 1;
-    double np = yp * yp, nq = yq * yq;
-#pragma unroll
-    for (int o = 1; o < (1 << LC); o <<= 1) {
-        np += __shfl_xor_sync(full, np, o);
-        nq += __shfl_xor_sync(full, nq, o);
-    }
+    const double np = row_dot_warp<LC>(yp, yp, lane), nq = row_dot_warp<LC>(yq, yq, lane);
     // one root per lane (its lowest bit: the row), passed to the other
     const double nm = (lane & 1) ? nq : np, im = nm > 1e-290 ? rsqrt64(nm) : 0.0, sm = nm * im;
     const double io = __shfl_xor_sync(full, im, 1), so = __shfl_xor_sync(full, sm, 1);
@@ -1667,7 +1702,7 @@ __device__ __forceinline__ void svd_place_warp(double yp, double yq, double &sp,
     sq = (lane & 1) ? sm : so;
     ip = (lane & 1) ? io : im;
     iq = (lane & 1) ? im : io;
-    // (non-negative: ordered as their bits; equal ones in the order of the halves)
+    // (non-negative: ordered as their bits; equal ones in row order)
     const long long a = __double_as_longlong(sp), b = __double_as_longlong(sq);
     const long long c = __shfl_xor_sync(full, a, 1 << LC), d = __shfl_xor_sync(full, b, 1 << LC);
     pp = (b > a) + (c > a || (second && c == a)) + (d > a || (second && d == a));
@@ -1700,13 +1735,9 @@ __global__ void __launch_bounds__(32 * E64W_WARPS) k_estimate_f64w(GsProblem P, 
     // column (lane & 15) of the unfolding; the half's first row pair
     const int col = lane & 15, h = lane >> 4;
     double yp = a[32 * h + col], yq = a[32 * h + 16 + col], zp = 2 * h == col, zq = 2 * h + 1 == col;
-    double tot = fabs(yp) + fabs(yq);
-    double high = h || (col >> 2) >= 2 || (col & 3) >= 2 ? tot : 0.0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        tot += __shfl_xor_sync(full, tot, o);
-        high += __shfl_xor_sync(full, high, o);
-    }
+    const double both = __dadd_rn(fabs(yp), fabs(yq));
+    const double high = entry_sum_warp(h || (col >> 2) >= 2 || (col & 3) >= 2 ? both : 0.0);
+    const double tot = entry_sum_warp(both);
     double b[6] = {0, 0, 0, high, 0, 0}, rrel = 1e30;
     if (tot != 0.0) {
         double sp, sq, ip, iq;
@@ -1765,33 +1796,25 @@ __global__ void __launch_bounds__(32 * E64W_WARPS) k_estimate_f64w(GsProblem P, 
         const double lo2 = __shfl_xor_sync(full, lo, 4), hi2 = __shfl_xor_sync(full, hi, 4);
         double mn, mx;
         product_range(lo, hi, lo2, hi2, mn, mx);
-        double Myz = l < ji ? dl * mx : 0.0, myz = l < ji ? dl * mn : 0.0;
-#pragma unroll
-        for (int o = 1; o < 4; o <<= 1) {
-            Myz += __shfl_xor_sync(full, Myz, o);
-            myz += __shfl_xor_sync(full, myz, o);
-        }
+        const double Myz = quad_sum(l < ji ? __dmul_rn(dl, mx) : 0.0);
+        const double myz = quad_sum(l < ji ? __dmul_rn(dl, mn) : 0.0);
         product_range(lx, hx, myz, Myz, mn, mx);
-        double M = i < jr ? si * mx : 0.0, m = i < jr ? si * mn : 0.0;
-#pragma unroll
-        for (int o = 8; o < 32; o <<= 1) {
-            M += __shfl_xor_sync(full, M, o);
-            m += __shfl_xor_sync(full, m, o);
+        double M = 0.0, m = 0.0;
+        for (int ii = 0; ii < jr; ii++) {
+            M = fma(s[ii], __shfl_sync(full, mx, 8 * ii), M);
+            m = fma(s[ii], __shfl_sync(full, mn, 8 * ii), m);
         }
-        // residual: the lane's entries (x, y, z) = (lane >> 3, (lane >> 1) & 3, 2 (lane & 1) + {0, 1})
-        const int rx = lane >> 3, ry = (lane >> 1) & 3, rz = 2 * (lane & 1);
-        double r0 = a[2 * lane], r1 = a[2 * lane + 1];
+        // residual: the lane's entries of its first layout
+        double r0 = a[32 * h + col], r1 = a[32 * h + 16 + col];
         for (int ii = 0; ii < jr; ii++)
             for (int k = 0; k < 4; k++) {
                 const double sd = s_sd[wl][ii][k];
                 if (sd == 0.0) break;   // past the kept terms
-                const double sab = sd * s_u[wl][ii][rx] * s_W[wl][ii][k][ry];
-                r0 = fma(-sab, s_V[wl][ii][k][rz], r0);
-                r1 = fma(-sab, s_V[wl][ii][k][rz + 1], r1);
+                const double xw = sd * s_V[wl][ii][k][col & 3] * s_W[wl][ii][k][col >> 2];
+                r0 = fma(-s_u[wl][ii][2 * h], xw, r0);
+                r1 = fma(-s_u[wl][ii][2 * h + 1], xw, r1);
             }
-        double sr = fabs(r0) + fabs(r1);
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) sr += __shfl_xor_sync(full, sr, o);
+        const double sr = entry_sum_warp(__dadd_rn(fabs(r0), fabs(r1)));
         b[0] = m - sr;
         b[1] = M + sr;
         b[2] = sr;

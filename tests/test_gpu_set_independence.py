@@ -1,6 +1,7 @@
 """A cube's or a point's result does not depend on what else is in the call:
 the same tensors whatever the number of octets in a launch (one warp per
-octet, or a block's four when there are few)."""
+octet, or a block's four when there are few), the same bounds whatever the
+length of the list (one warp per cube, or four lanes in longer ones)."""
 import numpy as np
 import pytest
 
@@ -39,3 +40,32 @@ def test_tensors_of_a_set_and_its_parts(level, atoms):
     Ap, _, _ = _parts(xyz, r, keys, (1, 90, 608))
     assert np.abs(A).sum() > 0
     assert np.array_equal(A, Ap)
+
+
+@pytest.mark.parametrize("level", [0, 1, 2, 3])
+@pytest.mark.parametrize("atoms", [5, 600])
+def test_bounds_of_a_set_and_its_parts(level, atoms):
+    xyz, r = synth.globular(atoms, seed=32)
+    keys = _keys(xyz, r, level, 600, seed=10 + level)   # 4800 cubes (an octet of eight per key), seven invalid of eight
+    _, b, d = gs.gs_cube_decisions(xyz, r, D, C, PREC, EDGE, DEPTH, keys)
+    _, bp, dp = _parts(xyz, r, keys, (1, 60, 252, 444))   # up to 1536 cubes each
+    assert len(np.unique(b[:, 4:], axis=0)) > 1   # several ranks
+    assert np.array_equal(b, bp) and np.array_equal(d, dp)
+
+
+@pytest.mark.parametrize("case", ["one", "line", "cross"])
+def test_bounds_of_symmetric_tensors(case):
+    """equal singular values and exact zeros: cubes centred on an atom, or
+    with atoms placed symmetrically about them"""
+    xyz = {"one": [[0.0, 0.0, 0.0]], "line": [[-1.0, 0.0, 0.0], [1.0, 0.0, 0.0]],
+           "cross": [[-1.0, 0.0, 0.0], [1.0, 0.0, 0.0], [0.0, -1.0, 0.0], [0.0, 1.0, 0.0], [0.0, 0.0, -1.0],
+                     [0.0, 0.0, 1.0]]}[case]
+    xyz = np.array(xyz)
+    r = np.full(len(xyz), 1.5)
+    o, nroot, _ = oracle.root_grid(xyz, r, D, C, EDGE, DEPTH)
+    # on the lattice's own planes and between them
+    xyz = xyz + (np.asarray(o) + np.floor((0.5 - np.asarray(o)) / 0.125) * 0.125)
+    keys = np.concatenate([_keys(xyz, r, 3, 400, seed=5), _keys(xyz, r, 2, 300, seed=6)])
+    A, b, d = gs.gs_cube_decisions(xyz, r, D, C, PREC, EDGE, DEPTH, keys)
+    Ap, bp, dp = _parts(xyz, r, keys, range(50, 700, 50))
+    assert np.array_equal(A, Ap) and np.array_equal(b, bp) and np.array_equal(d, dp)
