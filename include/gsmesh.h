@@ -244,7 +244,9 @@ int mesh_gaussian_surface_into(const double *atoms, const double *radii, int64_t
  *   D [n_mols] host.  Atoms and radii host or device.
  * opt->batch_mode:
  *   GS_BATCH_SHARED_LEVELS (default; GS_CHILD_REPROJECT only, else as
- *   GS_BATCH_THREADS): the molecules are grouped by D.  Per group one level
+ *   GS_BATCH_THREADS): the molecules are grouped by D and by what their
+ *   largest cutoff radius selects in the tensor accumulation (intervals of
+ *   an eighth of an octave on every level).  Per group one level
  *   loop (section 2.2) runs each kernel of a level once over the octets of
  *   all its molecules; every octet carries its molecule's index, and a
  *   device table holds each molecule's atoms, cell list and root grid.  The

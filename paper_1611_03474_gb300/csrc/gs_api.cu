@@ -1212,8 +1212,8 @@ extern "C" int mesh_gaussian_surface_into(const double *atoms, const double *rad
 
 // ---- the batched form
 
-// the level loop of a group of molecules sharing D (section 2.2, steps 1-3,
-// for all of them at once): each kernel of a level runs once over the
+// the level loop of a group of molecules sharing D and the class of their 1-D
+// coefficients on every level (section 2.2, steps 1-3, for all of them at once): each kernel of a level runs once over the
 // octets of every molecule of the group.  On return pm[mols[g]] holds the
 // molecule's accepted cubes, in the order its own level loop gives them,
 // and its level statistics.
@@ -1242,12 +1242,11 @@ static int group_levels(const std::vector<int64_t> &mols, std::vector<PreMol> &p
     GS_CHECK(cudaMemsetAsync(d_cnt, 0, GS_NCNT * sizeof(unsigned long long), st));
     GS_CHECK(cudaMemcpyAsync(d_probs, hp.data(), sizeof(GsProblem) * (size_t)G, cudaMemcpyHostToDevice, st));
     // the record the shared kernels read: the group's common scalars (D, c,
-    // precision, depth, order, norm); level-0 children outside a molecule's
+    // precision, depth, order, norm) and a cutoff radius of the group's
+    // coefficient class; level-0 children outside a molecule's
     // root grid are masked explicitly, so its root extent is unbounded
     GsProblem P0 = hp[0];
     for (int a = 0; a < 3; a++) P0.nroot[a] = (int64_t)1 << 40;
-    // the 1-D coefficients must hold for the largest cutoff radius of them all
-    for (int g = 1; g < G; g++) P0.pad = std::max(P0.pad, hp[(size_t)g].pad);
     P0.near = d_near;
     uint64_t *parents = nullptr;
     uint8_t *vmask0 = nullptr;
@@ -1531,23 +1530,42 @@ static int batch_shared(const double *atoms, const double *radii, const int64_t 
                 if (rc) bad = m;
             }
         }
-        if (!rc) {
+        // one level loop per coefficient class, so that each molecule's tensors
+        // are those of its own call (nearly always one class: cubes of 2 to 0.25
+        // A at D = 0.5 have one for largest radii of 1.5 to 1.8 A)
+        std::vector<std::vector<int>> classes;
+        std::vector<std::vector<int64_t>> parts;
+        if (!rc)
+            for (int64_t m : groups[(size_t)k]) {
+                std::vector<int> cl;
+                for (int l = 0; l <= max_depth; l++) cl.push_back(gs_coeff_class(pm[(size_t)m].PR.P, l));
+                size_t i = (size_t)(std::find(classes.begin(), classes.end(), cl) - classes.begin());
+                if (i == classes.size()) {
+                    classes.push_back(cl);
+                    parts.emplace_back();
+                }
+                parts[i].push_back(m);
+            }
+        for (const auto &part : parts) {
             bool retry = false;
-            rc = group_levels(groups[(size_t)k], pm, base, max_depth, st, (int64_t)1 << 21, &retry);
+            rc = group_levels(part, pm, base, max_depth, st, (int64_t)1 << 21, &retry);
             if (rc && retry) {
                 cudaGetLastError();
-                rc = group_levels(groups[(size_t)k], pm, base, max_depth, st, (int64_t)1 << 18, nullptr);
+                rc = group_levels(part, pm, base, max_depth, st, (int64_t)1 << 18, nullptr);
                 if (!rc)
-                    for (int64_t m : groups[(size_t)k]) pm[(size_t)m].lv.retries = 1;
+                    for (int64_t m : part) pm[(size_t)m].lv.retries = 1;
             }
-        }
-        if (!rc) {
-            cudaError_t e = gs_sync(st);
-            if (e != cudaSuccess) rc = gs_fail_cuda(e, "batch levels", __FILE__, __LINE__);
+            if (!rc) {
+                cudaError_t e = gs_sync(st);
+                if (e != cudaSuccess) rc = gs_fail_cuda(e, "batch levels", __FILE__, __LINE__);
+            }
+            if (rc) break;
+            std::lock_guard<std::mutex> lk(mu);
+            ready.insert(ready.end(), part.begin(), part.end());
+            cv.notify_all();
         }
         if (rc) { fail(rc, bad); }
         std::lock_guard<std::mutex> lk(mu);
-        if (!rc) ready.insert(ready.end(), groups[(size_t)k].begin(), groups[(size_t)k].end());
         groups_left--;
         cv.notify_all();
     };

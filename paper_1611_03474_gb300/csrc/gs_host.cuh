@@ -31,6 +31,9 @@ int gs_gather_atoms(const int32_t *d_perm, int64_t n, const double *d_xyz, const
 
 // gs_level.cu
 int gs_quadrature_init(void);
+// what the 1-D coefficients of a level depend on beside D and the cube edge:
+// problems that agree in these three get the same coefficients, bit for bit
+int gs_coeff_class(const GsProblem &P, int level);
 // ev (nullable): two events recorded before and after the launch
 // accumulate A for the 8 children of each parent (level-1 coords in parents,
 // or the implicit root blocks when parents == NULL); vmask (nullable) selects

@@ -149,6 +149,31 @@ struct Series {
     double kappa;               // mu = kappa m
     double c[4][SERIES_MAX];
 };
+// B = 2^(e/8), on a fixed scale of eight steps per octave: inputs that differ
+// a little in their largest radius share the polynomials
+#define SERIES_NONE (1 << 20)
+static int series_scale(double D, double hh, double R)
+{
+    const double bmax = 2.0 * D * hh * (R + hh);
+    if (!(D * hh * hh <= 4.0) || !(bmax <= 14.0) || !(bmax > 1e-30)) return SERIES_NONE;
+    return (int)ceil(8.0 * log2(bmax));
+}
+// exp(-D m^2) stays in gs_exp's range for |m| <= R + 3 hh
+static bool series_range64(const GsProblem &P, double hh)
+{
+    return P.D * (P.pad + 3.0 * hh) * (P.pad + 3.0 * hh) <= 690.0;
+}
+// exp(-D m^2) stays above the flush range (2^-126) for every atom that
+// reaches an interval
+static bool series_range32(const GsProblem &P, double hh)
+{
+    return P.D * (P.pad + hh) * (P.pad + hh) <= 85.0;
+}
+int gs_coeff_class(const GsProblem &P, int level)
+{
+    const double hh = 0.5 * gs_h(P, level);
+    return 4 * series_scale(P.D, hh, P.pad) + (series_range64(P, hh) ? 2 : 0) + (series_range32(P, hh) ? 1 : 0);
+}
 static int series_coeffs(double D, double hh, double R, double tol, const int *Ks, int nK, Series *out)
 {
     constexpr int NT = 48;
@@ -166,11 +191,9 @@ static int series_coeffs(double D, double hh, double R, double tol, const int *K
                     T[n][i] = (i > 0 ? 4.0 * T[n - 1][i - 1] : 0.0) - 2.0 * T[n - 1][i] - T[n - 2][i];
         }
     } tab;
-    const double a2 = D * hh * hh, bmax = 2.0 * D * hh * (R + hh);
-    if (!(a2 <= 4.0) || !(bmax <= 14.0) || !(bmax > 1e-30)) return 0;
-    // B on a fixed scale of eight steps per octave: inputs that differ a
-    // little in their largest radius share the polynomials
-    const double B = exp2(ceil(8.0 * log2(bmax)) / 8.0), B2 = B * B;
+    const int scale = series_scale(D, hh, R);
+    if (scale == SERIES_NONE) return 0;
+    const double a2 = D * hh * hh, B = exp2(scale / 8.0), B2 = B * B;
     double t[4][NT];
     int N = 0;
     double f = 1.0;             // B^(2k) / (2k)!
@@ -333,7 +356,8 @@ struct Series64 {
 // every entry adds them in that order in either form, so a cube's tensor
 // does not depend on how many octets share its launch.
 // BATCH: octet o belongs to molecule mol[o], whose problem is probs[mol[o]]
-// (the molecules of one launch share D, so one quadrature rule serves all)
+// (the molecules of one launch share D and the coefficient class, so one set
+// of polynomials or one quadrature rule serves all)
 template <class C, bool BATCH>
 __global__ void __launch_bounds__(32 * ACC_WARPS) k_accum_f64(const __grid_constant__ GsProblem P0, int level,
                                                                const uint64_t *parents, const uint8_t *vmask,
@@ -594,8 +618,7 @@ int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const
     static const int Ks[] = {7, 8, 9, 10, 12, 15, 20};
     Series S;
     int K = 0;
-    // exp(-D m^2) stays in gs_exp's range for |m| <= R + 3 hh
-    if (P.D * (P.pad + 3.0 * hh) * (P.pad + 3.0 * hh) <= 690.0) K = series_coeffs(P.D, hh, P.pad, 1e-15, Ks, 7, &S);
+    if (series_range64(P, hh)) K = series_coeffs(P.D, hh, P.pad, 1e-15, Ks, 7, &S);
 #define GS_ACC64(K_)                                                                                                    case K_: {                                                                                                              Series64<K_> c;                                                                                                     c.kappa = S.kappa;                                                                                                  for (int q = 0; q < 4; q++) memcpy(c.c[q], S.c[q], sizeof(double) * K_);                                            run(c);                                                                                                             break;                                                                                                          }
     switch (K) {
         GS_ACC64(7) GS_ACC64(8) GS_ACC64(9) GS_ACC64(10) GS_ACC64(12) GS_ACC64(15) GS_ACC64(20)
@@ -2498,9 +2521,7 @@ int gs_accum_f32(const GsProblem &P, int level, const uint64_t *d_parents, const
     static const int Ks[] = {5, 6, 8, 11, 14};
     Series S;
     int K = 0;
-    // exp(-D m^2) stays above the flush range (2^-126) for every atom that
-    // reaches an interval
-    if (P.D * (P.pad + hh) * (P.pad + hh) <= 85.0) K = series_coeffs(P.D, hh, P.pad, 2e-8, Ks, 5, &S);
+    if (series_range32(P, hh)) K = series_coeffs(P.D, hh, P.pad, 2e-8, Ks, 5, &S);
     int rc;
 #define GS_ACC32(K_)                                                                                                    case K_: {                                                                                                              Series32<K_> c;                                                                                                     c.kappa = (float)S.kappa;                                                                                           for (int q = 0; q < 4; q++)                                                                                             for (int k = 0; k < K_; k++) c.c[q][k] = make_float2((float)S.c[q][k], (float)S.c[q][k]);                       rc = run("k_accum_f32<series" #K_ ">", c);                                                                         break;                                                                                                          }
     switch (K) {

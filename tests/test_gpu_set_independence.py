@@ -1,7 +1,8 @@
 """A cube's or a point's result does not depend on what else is in the call:
 the same tensors whatever the number of octets in a launch (one warp per
 octet, or a block's four when there are few), the same bounds whatever the
-length of the list (one warp per cube, or four lanes in longer ones)."""
+length of the list (one warp per cube, or four lanes in longer ones), and the same cubes in a
+batch as alone, also where a decision is a tie."""
 import numpy as np
 import pytest
 
@@ -69,3 +70,36 @@ def test_bounds_of_symmetric_tensors(case):
     A, b, d = gs.gs_cube_decisions(xyz, r, D, C, PREC, EDGE, DEPTH, keys)
     Ap, bp, dp = _parts(xyz, r, keys, range(50, 700, 50))
     assert np.array_equal(A, Ap) and np.array_equal(b, bp) and np.array_equal(d, dp)
+
+
+def _bound_ties(seed, which):
+    """An atom in the root cube [0, 2]^3 and the isovalue equal to that
+    cube's own bound L or U as gs_cube_decisions gives it."""
+    rng = np.random.default_rng(seed)
+    xyz, r = rng.uniform(0.1, 1.9, (1, 3)), np.array([1.5])
+    c = 1.0
+    for _ in range(3):   # the tensor depends on c through nothing but the lattice's origin
+        o, _, _ = oracle.root_grid(xyz, r, D, c, EDGE, DEPTH)
+        q = [int(round(-x / 2.0)) for x in o]
+        key = np.array([q[0] | q[1] << 18 | q[2] << 36 | 30 << 54], dtype=np.uint64)
+        _, b, _ = gs.gs_cube_decisions(xyz, r, D, c, PREC, EDGE, DEPTH, key)
+        last, c = c, float(b[0, which])
+    assert c == last
+    return xyz, r, c
+
+
+@pytest.mark.parametrize("mode", ["GS_PREC_FP64", "GS_PREC_MIXED"])
+@pytest.mark.parametrize("which", [0, 1])
+def test_ties_in_a_batch(mode, which):
+    """beside a molecule whose larger cutoff radius selects other polynomials"""
+    other = (np.array([[0.0, 0.0, 0.0], [1.5, 0.3, 0.2]]), np.array([2.6, 1.2]), D)
+    kw = dict(min_edge=EDGE, precision_mode=getattr(gs, mode))
+    for seed in range(12):
+        xyz, r, c = _bound_ties(seed, which)
+        one = gs.mesh_gaussian_surface(xyz, r, D, c, PREC, DEPTH, **kw)
+        assert one.stats["near_threshold"][0] >= 1
+        b = gs.mesh_gaussian_surface_batch([other, (xyz, r, D)], c, PREC, DEPTH, **kw)[1]
+        for k in ("examined", "discarded", "accepted", "forced", "split"):
+            assert b.stats[k] == one.stats[k], k
+        assert np.array_equal(b.cube_keys, one.cube_keys)
+        assert np.array_equal(b.vertices, one.vertices) and np.array_equal(b.triangles, one.triangles)
