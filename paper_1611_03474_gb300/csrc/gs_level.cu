@@ -1287,6 +1287,19 @@ __device__ __forceinline__ double entry_sum(const double (&v)[4][4])
     return __dadd_rn(t[0], t[1]);
 }
 
+// Squares of the entries and their products leave FP64's range for isovalues
+// below about 1e-130: a tensor whose sum of magnitudes lies outside 2^-300 ..
+// 2^300 is scaled by a power of two (exactly), and its bounds scaled back.
+// False: no scaling, and both factors are 1.
+__device__ __forceinline__ bool svd_scale64(double tot, double &to, double &back)
+{
+    const int e = (__double2hiint(tot) >> 20) & 0x7ff;
+    const bool out = (e < 723 || e > 1323) && tot != 0.0 && e < 2046;
+    to = out ? __hiloint2double((2046 - (e ? e : 1)) << 20, 0) : 1.0;
+    back = out ? __hiloint2double((e ? e : 1) << 20, 0) : 1.0;
+    return out;
+}
+
 // one-sided Jacobi on the 4 rows of a matrix whose columns lie in the four
 // lanes of a quad (NC each): y the lane's columns, z its column of the
 // accumulated rotations (initially the identity).  Each of the three rounds
@@ -1530,6 +1543,13 @@ __global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, co
                 if (l < 2) v[j][k] = 0.0;
         high = quad_sum(entry_sum(v));
     }
+    double to, back;
+    const bool scaled = __any_sync(full, svd_scale64(tot, to, back));
+    if (scaled)
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+#pragma unroll
+            for (int k = 0; k < 4; k++) y[j][k] *= to;
     double s[4], rm = 0.0, rrel = 1e30;
     jacobi_quad<4>(y, z, true, lane);
     svd_order_quad<4>(y, z, s, lane);
@@ -1544,6 +1564,11 @@ __global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, co
     for (int j = 0; j < 4; j++)
 #pragma unroll
         for (int k = 0; k < 4; k++) R[j][k] = q >= 0 ? a[16 * j + 4 * k] : 0.0;
+    if (scaled)
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+#pragma unroll
+            for (int k = 0; k < 4; k++) R[j][k] *= to;
     double lx, hx;   // lane l: the range of u_l
     {
         double cf[4];
@@ -1613,7 +1638,7 @@ __global__ void __launch_bounds__(128) k_estimate_f64(GsProblem P, int level, co
         for (int k = 0; k < 4; k++) R[j][k] = fabs(R[j][k]);
     const double sr = quad_sum(entry_sum(R));
     if (q < 0 || l != 0) return;
-    const double b[6] = {m - sr, M + sr, sr, high, (double)jr, (double)inner};
+    const double b[6] = {(m - sr) * back, (M + sr) * back, sr * back, high, (double)jr, (double)inner};
     finish_f64(P, level, q, a, b, rrel, dec, bounds);
 }
 
@@ -1763,8 +1788,13 @@ __global__ void __launch_bounds__(32 * E64W_WARPS) k_estimate_f64w(GsProblem P, 
     const double tot = entry_sum_warp(both);
     double b[6] = {0, 0, 0, high, 0, 0}, rrel = 1e30;
     if (tot != 0.0) {
-        double sp, sq, ip, iq;
+        double sp, sq, ip, iq, to, back;
         int pp, pq;
+        const bool scaled = svd_scale64(tot, to, back);
+        if (scaled) {
+            yp *= to;
+            yq *= to;
+        }
         jacobi_warp<4>(yp, yq, zp, zq, lane);
         svd_place_warp<4>(yp, yq, sp, sq, ip, iq, pp, pq, lane);
         s_V[wl][pp][col >> 2][col & 3] = yp * ip;
@@ -1829,6 +1859,10 @@ __global__ void __launch_bounds__(32 * E64W_WARPS) k_estimate_f64w(GsProblem P, 
         }
         // residual: the lane's entries of its first layout
         double r0 = a[32 * h + col], r1 = a[32 * h + 16 + col];
+        if (scaled) {
+            r0 *= to;
+            r1 *= to;
+        }
         for (int ii = 0; ii < jr; ii++)
             for (int k = 0; k < 4; k++) {
                 const double sd = s_sd[wl][ii][k];
@@ -1838,9 +1872,9 @@ __global__ void __launch_bounds__(32 * E64W_WARPS) k_estimate_f64w(GsProblem P, 
                 r1 = fma(-s_u[wl][ii][2 * h + 1], xw, r1);
             }
         const double sr = entry_sum_warp(__dadd_rn(fabs(r0), fabs(r1)));
-        b[0] = m - sr;
-        b[1] = M + sr;
-        b[2] = sr;
+        b[0] = (m - sr) * back;
+        b[1] = (M + sr) * back;
+        b[2] = sr * back;
         b[4] = (double)jr;
         b[5] = (double)inner;
     }
