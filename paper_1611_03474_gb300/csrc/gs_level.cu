@@ -2280,7 +2280,7 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 4) k_accum_f32(const __grid_co
     const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
     const int oWXY = ACF_WXY + ((cy * 2 + cx) * 4 + j) * 4, oZ = ACF_Z + 8 * cz;
     const float nDl2e = (float)(-P0.D * 1.4426950408889634);
-    const float hh = 0.5f * hf;
+    const float hh = 0.5f * hf, ctol = fmaxf(1e-5f, 4e-7f * hf);
     for (int64_t o = (int64_t)blockIdx.x * ACC_WARPS + wl; o < n_oct; o += (int64_t)gridDim.x * ACC_WARPS) {
         const GsProblem &P = BATCH ? probs[mol[o]] : P0;
         Octet q = octet_of(P, level, parents, vmask, o);
@@ -2424,9 +2424,11 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 4) k_accum_f32(const __grid_co
         // membership of one candidate per lane (i < 0: none): FP32 box
         // distance with a relative margin, the exact FP64 test inside the
         // margin; members join the atom queue.  Per axis both gaps follow from
-        // u = e_1 - x; t = d^2 - (R^2 - tol) of a child is negative for a
-        // member, and as unsigned bits at most those of 2 tol inside the
-        // margin
+        // u = e_1 - x, whose rounding (1.3e-7 h with that of h) moves a squared
+        // gap by up to 2.6e-7 h R <= 1.3e-7 h (R^2 + 1): the margin 1e-5 (R^2 + 1)
+        // covers it up to h = 25 A, 4e-7 h (R^2 + 1) beyond.  t = d^2 - (R^2 -
+        // tol) of a child is negative for a member, and as unsigned bits at
+        // most those of 2 tol inside the margin
         auto filter = [&](int i) {
             unsigned m = 0;
             if (i >= 0) {
@@ -2440,7 +2442,7 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 4) k_accum_f32(const __grid_co
                     g2[a][1] = g1 * g1;
                 }
                 const float R2 = P.fR2[i];
-                const float tol = 1e-5f * R2 + 1e-5f, lo = R2 - tol;
+                const float tol = ctol * R2 + ctol, lo = R2 - tol;
                 unsigned tb[8], nmin = 0xffffffffu;
 #pragma unroll
                 for (int cc = 0; cc < 8; cc++) {
