@@ -1119,7 +1119,10 @@ __device__ __forceinline__ void trilinear_range(const T *a, T high, T &mn, T &mx
     mn = lo - high;
     mx = hi + high;
 }
-// squared distance from the rank-one tensor; a[0] != 0
+// squared distance from the rank-one tensor; a[0] != 0.  Its squares lose
+// their precision below 1e-38 (FP32) and 1e-308 (FP64), so it is compared only
+// with the square of a room above 1e-17 or 1e-150 (at an isovalue of 1e-20 the
+// FP32 form otherwise drops cubes that the SVD keeps)
 template <typename T>
 __device__ __forceinline__ T rank_one_dist2(const T *a)
 {
@@ -1940,7 +1943,7 @@ __global__ void __launch_bounds__(256) k_estimate_pre64(GsProblem P, int level, 
                 trilinear_range<double>(a, high, mn, mx);
                 const double room = fmax(P.c - mx, mn - P.c) - 1e-8 * (P.c + tot);
                 slow = true;
-                if (room > 0.0 && fabs(a[0]) > 1e-3 * tot &&
+                if (room > 1e-150 && fabs(a[0]) > 1e-3 * tot &&
                     RANK_ONE_SLOPE * RANK_ONE_SLOPE * rank_one_dist2<double>(a) < room * room) {
                     dec[q] = DEC_DISCARD;
                     slow = false;
@@ -2653,7 +2656,7 @@ __device__ __forceinline__ bool estimate_fast_f32(const GsProblem &P, int level,
         float mn, mx;
         trilinear_range<float>(a, high, mn, mx);
         const float room = fmaxf(c - mx, mn - c) - cm - RANK_ONE_SLOPE * (8.f * dA + 1e-6f * tot);
-        if (!(room > 0.f && fabsf(a[0]) > 1e-3f * tot &&
+        if (!(room > 1e-17f && fabsf(a[0]) > 1e-3f * tot &&
               1.0001f * (RANK_ONE_SLOPE * RANK_ONE_SLOPE) * rank_one_dist2<float>(a) < room * room))
             return false;
         if (why_cnt) atomicAdd(&why_cnt[10], 1ull);   // decided without the SVD
