@@ -869,7 +869,7 @@ __global__ void __launch_bounds__(32 * FD_WARPS) k_field_adjoint(const __grid_co
     const unsigned below = (1u << lane) - 1u;
     const int64_t k = (int64_t)blockIdx.x * FD_WARPS + w;
     if (k >= V.n) return;
-    const double x = V.ax[k], y = V.ay[k], z = V.az[k], R2 = V.aR2[k], nD = -V.D;
+    const double x = V.ax[k], y = V.ay[k], z = V.az[k], R2 = V.aR2[k], nD = -V.D, r = V.ar[k];
     const float c[3] = {V.hx[k], V.hy[k], V.hz[k]};
     // FP32 screen: offsets rounded to 6e-8 of their size on both sides
     const float ext = fmaxf(fabsf(c[0]), fmaxf(fabsf(c[1]), fabsf(c[2]))) + V.pad_f;
@@ -887,7 +887,7 @@ __global__ void __launch_bounds__(32 * FD_WARPS) k_field_adjoint(const __grid_co
             sx = fma(s, dx, sx);
             sy = fma(s, dy, sy);
             sz = fma(s, dz, sz);
-            s2 = fma(s, d2, s2);
+            s2 = fma(s, fma(-r, r, d2), s2);   // (d^2 - r^2 by term: the two sums would nearly cancel for a large r)
         }
         __syncwarp();
     };
@@ -925,13 +925,13 @@ __global__ void __launch_bounds__(32 * FD_WARPS) k_field_adjoint(const __grid_co
         s2 += __shfl_xor_sync(full, s2, o);
     }
     if (lane == 0 && (s0 != 0.0 || s2 != 0.0 || sx != 0.0 || sy != 0.0 || sz != 0.0)) {
-        const double wt = V.aw[k], r = V.ar[k], f = 2.0 * V.D * wt;
+        const double wt = V.aw[k], f = 2.0 * V.D * wt;
         const int64_t o = perm[k];
         atomicAdd(&gx[3 * o], f * sx);
         atomicAdd(&gx[3 * o + 1], f * sy);
         atomicAdd(&gx[3 * o + 2], f * sz);
         atomicAdd(&gr[o], f * r * s0);
-        atomicAdd(gD, -wt * fma(-r * r, s0, s2));
+        atomicAdd(gD, -wt * s2);
     }
 }
 
