@@ -17,6 +17,9 @@
 //   capacity@L  the level loop reports a full internal table at level L on
 //               the call's first attempt (the call retries with smaller
 //               level chunks, as for a real overflow)
+//   staging     the triangulation finds no room for its staging slots
+//   pool@C      the triangulation's pool has room for C triangles and points
+//               (0: there is no pool)
 //   timeout     the call's first host wait times out (GS_ERR_TIMEOUT)
 #include <chrono>
 #include <cstdlib>
@@ -26,7 +29,7 @@
 #include "gs_host.cuh"
 
 namespace {
-enum FaultKind { F_NONE = 0, F_ALLOC = 1, F_CAPACITY = 2, F_TIMEOUT = 3 };
+enum FaultKind { F_NONE = 0, F_ALLOC = 1, F_CAPACITY = 2, F_TIMEOUT = 3, F_STAGING = 4, F_POOL = 5 };
 struct FaultState {
     int kind = F_NONE;
     long long arg = 0;
@@ -47,6 +50,11 @@ void gs_guard_begin(void)
     } else if (!strncmp(s, "capacity@", 9)) {
         g_fault.kind = F_CAPACITY;
         g_fault.arg = atoll(s + 9);
+    } else if (!strncmp(s, "pool@", 5)) {
+        g_fault.kind = F_POOL;
+        g_fault.arg = atoll(s + 5);
+    } else if (!strcmp(s, "staging")) {
+        g_fault.kind = F_STAGING;
     } else if (!strcmp(s, "timeout")) {
         g_fault.kind = F_TIMEOUT;
     }
@@ -65,6 +73,13 @@ bool gs_fault_capacity(int level)
     if (g_fault.kind != F_CAPACITY || g_fault.fired || level != g_fault.arg) return false;
     g_fault.fired = true;
     return true;
+}
+
+bool gs_fault_staging(void) { return g_fault.kind == F_STAGING; }
+
+int64_t gs_fault_pool(int64_t room)
+{
+    return g_fault.kind == F_POOL && g_fault.arg < room ? g_fault.arg : room;
 }
 
 static double wait_limit_s(void)

@@ -11,6 +11,8 @@ cudaError_t gs_sync(cudaStream_t st);
 void gs_guard_begin(void);
 bool gs_fault_alloc(void);
 bool gs_fault_capacity(int level);
+bool gs_fault_staging(void);
+int64_t gs_fault_pool(int64_t room);
 
 struct GsAtomsSoA {
     double *x, *y, *z, *r, *R2, *w;

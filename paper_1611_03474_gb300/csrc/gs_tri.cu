@@ -1344,34 +1344,14 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
     // staging slots; without room for them every cube is traced twice
     uint64_t *st_tri = nullptr, *st_pk = nullptr;
     double *st_xyz = nullptr;
-    if (cudaMallocAsync((void **)&st_tri, sizeof(uint64_t) * 3 * TRI_STAGE_T * (size_t)n, st) != cudaSuccess ||
+    if (gs_fault_staging() ||
+        cudaMallocAsync((void **)&st_tri, sizeof(uint64_t) * 3 * TRI_STAGE_T * (size_t)n, st) != cudaSuccess ||
         cudaMallocAsync((void **)&st_pk, sizeof(uint64_t) * TRI_STAGE_P * (size_t)n, st) != cudaSuccess ||
         cudaMallocAsync((void **)&st_xyz, sizeof(double) * 3 * TRI_STAGE_P * (size_t)n, st) != cudaSuccess) {
         cudaGetLastError();
         gs_free(st_tri, st); gs_free(st_pk, st); gs_free(st_xyz, st);
         st_tri = nullptr; st_pk = nullptr; st_xyz = nullptr;
     }
-    // and the pool for what the slots do not hold (on average less than one
-    // triangle and one point per cube); without it such cubes are traced twice
-    TriPool pool;
-    memset(&pool, 0, sizeof(pool));
-    if (st_tri && n < ((int64_t)1 << 28)) {   // (a place's halves stay below 2^32)
-        pool.cap = (unsigned)(n + 4096);
-        if (cudaMallocAsync((void **)&pool.tk, sizeof(uint64_t) * 3 * (size_t)pool.cap, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&pool.pk, sizeof(uint64_t) * (size_t)pool.cap, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&pool.xyz, sizeof(double) * 3 * (size_t)pool.cap, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&pool.off, sizeof(uint64_t) * (size_t)n, st) != cudaSuccess ||
-            cudaMallocAsync((void **)&pool.used, 2 * sizeof(unsigned long long), st) != cudaSuccess) {
-            cudaGetLastError();
-            gs_free(pool.tk, st); gs_free(pool.pk, st); gs_free(pool.xyz, st); gs_free(pool.off, st);
-            memset(&pool, 0, sizeof(pool));
-        } else {
-            cudaMemsetAsync(pool.used, 0, 2 * sizeof(unsigned long long), st);
-        }
-    }
-    auto free_pool = [&]() {
-        gs_free(pool.tk, st); gs_free(pool.pk, st); gs_free(pool.xyz, st); gs_free(pool.off, st); gs_free(pool.used, st);
-    };
     unsigned nb = (unsigned)((n + 127) / 128);
     // fold-root table; without room for it each cube solves its neighbours' roots
     uint8_t *fcount = nullptr;
@@ -1411,9 +1391,46 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
         gs_free(ntri, st); gs_free(npt, st); gs_free(tot, st);
         gs_free(st_tri, st); gs_free(st_pk, st); gs_free(st_xyz, st);
         gs_free(fcount, st); gs_free(froot, st);
-        free_pool();
         return rc;
     }
+    // and the pool for what the slots do not hold (on average less than one
+    // triangle and one point per cube); without it such cubes are traced
+    // twice.  It comes after the tables that spare more, and it is given back
+    // when a later allocation finds no room.
+    TriPool pool;
+    memset(&pool, 0, sizeof(pool));
+    auto drop_pool = [&]() {
+        gs_free(pool.tk, st); gs_free(pool.pk, st); gs_free(pool.xyz, st); gs_free(pool.off, st); gs_free(pool.used, st);
+        memset(&pool, 0, sizeof(pool));
+    };
+    const int64_t room = gs_fault_pool(n + 4096);
+    if (st_tri && n < ((int64_t)1 << 28) && room > 0) {   // (a place's halves stay below 2^32)
+        pool.cap = (unsigned)room;
+        if (cudaMallocAsync((void **)&pool.tk, sizeof(uint64_t) * 3 * (size_t)pool.cap, st) != cudaSuccess ||
+            cudaMallocAsync((void **)&pool.pk, sizeof(uint64_t) * (size_t)pool.cap, st) != cudaSuccess ||
+            cudaMallocAsync((void **)&pool.xyz, sizeof(double) * 3 * (size_t)pool.cap, st) != cudaSuccess ||
+            cudaMallocAsync((void **)&pool.off, sizeof(uint64_t) * (size_t)n, st) != cudaSuccess ||
+            cudaMallocAsync((void **)&pool.used, 2 * sizeof(unsigned long long), st) != cudaSuccess) {
+            cudaGetLastError();
+            drop_pool();
+        } else {
+            cudaMemsetAsync(pool.used, 0, 2 * sizeof(unsigned long long), st);
+        }
+    }
+    // once more without the pool when there is no room beside it: the cubes
+    // it held are then traced again at their final offsets
+    auto with_room = [&](auto step) {
+        int r = step();
+        if (r == GS_ERR_OOM && pool.tk) {
+            cudaGetLastError();
+            drop_pool();
+            r = step();
+        }
+        return r;
+    };
+    auto alloc = [&](auto **p, size_t count) {
+        return with_room([&]() { return gs_alloc((void **)p, sizeof(**p) * count, st); });
+    };
     if (order) {
         cudaMemsetAsync(ntri, 0, sizeof(int64_t) * (size_t)n, st);
         cudaMemsetAsync(npt, 0, sizeof(int64_t) * (size_t)n, st);
@@ -1425,8 +1442,8 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
     int64_t *mlist = nullptr;
     unsigned long long *nmlist = nullptr;
     if (X.mixed) {
-        rc = gs_alloc((void **)&mlist, sizeof(int64_t) * (size_t)n, st);
-        if (!rc) rc = gs_alloc((void **)&nmlist, sizeof(unsigned long long), st);
+        rc = alloc(&mlist, (size_t)n);
+        if (!rc) rc = alloc(&nmlist, 1);
         if (!rc) {
             cudaMemsetAsync(nmlist, 0, sizeof(unsigned long long), st);
             GS_LAUNCH(k_mixed_list, (unsigned)((n + 255) / 256), 256, 0, st)(X.mixed, n, mlist, nmlist);
@@ -1435,8 +1452,9 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
         }
     }
     gs_free(order, st);
-    rc = gs_scan_i64(ntri, n + 1, tot, st);
-    if (!rc) rc = gs_scan_i64(npt, n + 1, tot + 1, st);
+    // (a scan that finds no room leaves its values alone)
+    rc = with_room([&]() { return gs_scan_i64(ntri, n + 1, tot, st); });
+    if (!rc) rc = with_room([&]() { return gs_scan_i64(npt, n + 1, tot + 1, st); });
     int64_t h[2] = {0, 0};
     if (!rc) {
         cudaError_t e = cudaMemcpyAsync(h, tot, sizeof(h), cudaMemcpyDeviceToHost, st);
@@ -1444,15 +1462,15 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
         if (e != cudaSuccess) rc = gs_fail_cuda(e, "triangle counts", __FILE__, __LINE__);
     }
     if (!rc) {
-        rc = gs_alloc((void **)d_tri_keys, sizeof(uint64_t) * 3 * (size_t)(h[0] + 1), st);
-        if (!rc) rc = gs_alloc((void **)d_pt_keys, sizeof(uint64_t) * (size_t)(h[1] + 1), st);
-        if (!rc) rc = gs_alloc((void **)d_pt_xyz, sizeof(double) * 3 * (size_t)(h[1] + 1), st);
+        rc = alloc(d_tri_keys, 3 * (size_t)(h[0] + 1));
+        if (!rc) rc = alloc(d_pt_keys, (size_t)(h[1] + 1));
+        if (!rc) rc = alloc(d_pt_xyz, 3 * (size_t)(h[1] + 1));
     }
     if (!rc && st_tri) {
         int64_t *redo = nullptr;
         unsigned long long *nredo = nullptr;
-        rc = gs_alloc((void **)&redo, sizeof(int64_t) * (size_t)n, st);
-        if (!rc) rc = gs_alloc((void **)&nredo, sizeof(unsigned long long), st);
+        rc = alloc(&redo, (size_t)n);
+        if (!rc) rc = alloc(&nredo, 1);
         if (!rc) {
             cudaMemsetAsync(nredo, 0, sizeof(unsigned long long), st);
             GS_LAUNCH(k_tri_copy, nb, 128, 0, st)(n, pool, ntri, npt, st_tri, st_pk, st_xyz, *d_tri_keys, *d_pt_keys,
@@ -1473,7 +1491,7 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
             GS_LAUNCH(k_tri_emit<true>, nb, 128, 0, st)(X, ntri, npt, *d_tri_keys, *d_pt_keys, *d_pt_xyz,
                                                        d_counters + 1, mlist, nmlist);
     }
-    free_pool();
+    drop_pool();
     gs_free(mlist, st); gs_free(nmlist, st);
     gs_free(st_tri, st); gs_free(st_pk, st); gs_free(st_xyz, st);
     gs_free(fcount, st); gs_free(froot, st);
