@@ -1453,7 +1453,7 @@ int gs_triangulate(const TriCtx &X0, uint64_t **d_tri_keys, int64_t *ntri_total,
     }
     gs_free(order, st);
     // (a scan that finds no room leaves its values alone)
-    rc = with_room([&]() { return gs_scan_i64(ntri, n + 1, tot, st); });
+    if (!rc) rc = with_room([&]() { return gs_scan_i64(ntri, n + 1, tot, st); });
     if (!rc) rc = with_room([&]() { return gs_scan_i64(npt, n + 1, tot + 1, st); });
     int64_t h[2] = {0, 0};
     if (!rc) {

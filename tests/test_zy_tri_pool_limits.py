@@ -80,3 +80,16 @@ def test_failing_allocation_beside_the_pool(fault, make):
     # the tracing order's three are optional; the scans' two, the results' three and the redo list's two go on without the
     # pool
     assert served >= 3 + 7
+
+
+def test_failing_allocation_with_cubes_of_two_sizes(fault):
+    """(the list of the cubes with neighbours of another size among them)"""
+    xyz, r = synth.globular(14, seed=3)
+
+    def make():
+        return gs.mesh_gaussian_surface(xyz, r, 0.5, 1.0, 5e-2, 3)
+
+    ref = make()
+    assert ref.stats["mixed_cubes"] > 0
+    refused, served = _sweep(fault, make, ref)
+    assert refused > 50 and served >= 3 + 9
