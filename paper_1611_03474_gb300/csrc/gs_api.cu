@@ -347,7 +347,7 @@ struct LevelBatch {
 static int run_level(const GsProblem &P, int level, const uint64_t *d_parents, int64_t n_oct, int mode,
                      DevBufs &B, std::vector<uint64_t *> &acc_parts, std::vector<int64_t> &acc_counts,
                      uint64_t **d_next, int64_t *n_next, unsigned long long *d_counters, unsigned long long *d_pairs,
-                     unsigned long long *d_rechecked, unsigned long long *d_mism, bool both, unsigned *d_status,
+                     unsigned long long *d_rechecked, unsigned long long *d_mism, bool both,
                      gs_stats *stats, bool reexpand = false, const double *d_parA = nullptr,
                      double **d_nextA = nullptr, int64_t CH = (int64_t)1 << 21, LevelBatch *lb = nullptr)
 {
@@ -392,7 +392,7 @@ static int run_level(const GsProblem &P, int level, const uint64_t *d_parents, i
         int rc = gs_alloc((void **)&dec, (size_t)m * 8, st);
         if (rc) { drop_nexts(); return rc; }
         if (mode == GS_PREC_MIXED) {
-            rc = gs_level_mixed(P, level, par, m, dec, d_pairs, d_rechecked, d_mism, both, d_status, st,
+            rc = gs_level_mixed(P, level, par, m, dec, d_pairs, d_rechecked, d_mism, both, st,
                                 stats ? acc_ev.e : nullptr, d_mism + 1, probs, pmol, pvm);
         }
         double *dA = nullptr;
@@ -401,7 +401,7 @@ static int run_level(const GsProblem &P, int level, const uint64_t *d_parents, i
             if (rc) { gs_free(dec, st); drop_nexts(); return rc; }
             if (reexpand && d_parA) rc = gs_reexpand(d_parA + 64 * o0, m, dA, st);
             else
-                rc = gs_accum_f64(P, level, par, pvm, m, dA, d_pairs, d_status, st, stats ? acc_ev.e : nullptr, probs,
+                rc = gs_accum_f64(P, level, par, pvm, m, dA, d_pairs, st, stats ? acc_ev.e : nullptr, probs,
                                   pmol);
             if (!rc) rc = gs_estimate_f64(P, level, dA, m * 8, par, pvm, dec, nullptr, st);
         }
@@ -636,7 +636,7 @@ static int single_levels(const GsProblem &P, const gs_options &o, int max_depth,
         std::vector<int64_t> cnts;
         double *nextA = nullptr;
         rc = run_level(P, l, parents, n_oct, o.precision_mode, B, parts, cnts, &next, &nn, d_cnt, d_cnt + 8,
-                       d_cnt + 13, d_cnt + 14, (o.debug_flags & 1) != 0, d_status, stats, reexpand, parentA,
+                       d_cnt + 13, d_cnt + 14, (o.debug_flags & 1) != 0, stats, reexpand, parentA,
                        reexpand ? &nextA : nullptr, (o.debug_flags & 2) ? (int64_t)1000 : chunk);
         if (parentA) B.release(parentA);
         parentA = nextA;
@@ -1276,7 +1276,7 @@ static int group_levels(const std::vector<int64_t> &mols, std::vector<PreMol> &p
         uint64_t *next = nullptr;
         int64_t nn = 0;
         rc = run_level(P0, l, parents, n_oct, o.precision_mode, B, acc[(size_t)l], accn[(size_t)l], &next, &nn, d_cnt,
-                       d_cnt + 8, d_cnt + 13, d_cnt + 14, (o.debug_flags & 1) != 0, d_status, &gst, false, nullptr,
+                       d_cnt + 8, d_cnt + 13, d_cnt + 14, (o.debug_flags & 1) != 0, &gst, false, nullptr,
                        nullptr, (o.debug_flags & 2) ? (int64_t)1000 : CH, &lb);
         for (auto q : acc[(size_t)l]) B.keep(q);
         for (auto q : lb.acc_mol) B.keep(q);
@@ -2033,7 +2033,7 @@ extern "C" int gs_cube_decisions(const double *atoms, const double *radii, int64
             if (rc) break;
             cudaMemcpyAsync(dp, par.data(), sizeof(uint64_t) * (size_t)m, cudaMemcpyHostToDevice, st);
             cudaMemcpyAsync(dv, vm.data(), (size_t)m, cudaMemcpyHostToDevice, st);
-            rc = gs_accum_f64(PR.P, l, dp, dv, m, dA, nullptr, d_status, st);
+            rc = gs_accum_f64(PR.P, l, dp, dv, m, dA, nullptr, st);
             if (!rc) rc = gs_estimate_f64(PR.P, l, dA, m * 8, dp, dv, dd, dB, st);
             std::vector<double> tA((size_t)m * 8 * 64), tB((size_t)m * 8 * 6);
             std::vector<uint8_t> tD((size_t)m * 8);

@@ -44,13 +44,13 @@ int gs_coeff_class(const GsProblem &P, int level);
 // d_mol[o] whose problem is d_probs[d_mol[o]] (P then only supplies what the
 // molecules share: D, c, precision, the lattice spacing)
 int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const uint8_t *d_vmask, int64_t n_oct,
-                 double *d_A, unsigned long long *d_pairs, unsigned *d_status, cudaStream_t st, cudaEvent_t *ev = nullptr,
+                 double *d_A, unsigned long long *d_pairs, cudaStream_t st, cudaEvent_t *ev = nullptr,
                  const GsProblem *d_probs = nullptr, const int32_t *d_mol = nullptr);
 int gs_estimate_f64(const GsProblem &P, int level, const double *d_A, int64_t n_cubes, const uint64_t *d_parents,
                     const uint8_t *d_vmask, uint8_t *d_dec, double *d_bounds, cudaStream_t st);
 // mixed precision: FP32 accumulate (Kahan) + error bound, FP32 estimate with margins
 int gs_accum_f32(const GsProblem &P, int level, const uint64_t *d_parents, const uint8_t *d_vmask, int64_t n_oct,
-                 float *d_A, float *d_err, unsigned long long *d_pairs, unsigned *d_status, cudaStream_t st,
+                 float *d_A, float *d_err, unsigned long long *d_pairs, cudaStream_t st,
                  cudaEvent_t *ev = nullptr, unsigned long long *d_atom_octets = nullptr, const GsProblem *d_probs = nullptr,
                  const int32_t *d_mol = nullptr);
 int gs_estimate_f32(const GsProblem &P, int level, const float *d_A, const float *d_err, int64_t n_cubes,
@@ -89,7 +89,7 @@ int gs_reexpand(const double *d_Apar, int64_t n_oct, double *d_A, cudaStream_t s
 
 int gs_level_mixed(const GsProblem &P, int level, const uint64_t *d_parents, int64_t n_oct, uint8_t *d_dec,
                    unsigned long long *d_pairs, unsigned long long *d_rechecked, unsigned long long *d_mism,
-                   bool both, unsigned *d_status, cudaStream_t st, cudaEvent_t *ev = nullptr,
+                   bool both, cudaStream_t st, cudaEvent_t *ev = nullptr,
                    unsigned long long *d_why = nullptr, const GsProblem *d_probs = nullptr,
                    const int32_t *d_mol = nullptr, const uint8_t *d_vmask = nullptr);
 int gs_root_blocks(const GsProblem &P, uint64_t **d_keys, int64_t *n, cudaStream_t st);

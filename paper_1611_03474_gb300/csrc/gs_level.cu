@@ -24,14 +24,15 @@
 
 // ---------------------------------------------------------------- quadrature
 // Gauss-Legendre nodes t_k and folded weights W_kj = (2j+1)/2 * w_k * L_j(t_k),
-// so that alpha_j = sum_k W_kj f(t_k).  Variants with 8, 12, 16 and 24 nodes.
-#define GQ_VARIANTS 4
+// so that alpha_j = sum_k W_kj f(t_k) for j = 0, 1 (the end points give the
+// other two).  Variants with 8, 16 and 24 nodes.
+#define GQ_VARIANTS 3
 #define GQ_MAX 24
 __constant__ double c_gq_t[GQ_VARIANTS][GQ_MAX];
-__constant__ double c_gq_W[GQ_VARIANTS][GQ_MAX][4];
+__constant__ double c_gq_W[GQ_VARIANTS][GQ_MAX][2];
 __constant__ float c_gq_tf[GQ_VARIANTS][GQ_MAX];
-__constant__ float c_gq_Wf[GQ_VARIANTS][GQ_MAX][4];
-static const int kGqN[GQ_VARIANTS] = {8, 12, 16, 24};
+__constant__ float c_gq_Wf[GQ_VARIANTS][GQ_MAX][2];
+static const int kGqN[GQ_VARIANTS] = {8, 16, 24};
 
 // nodes of P_n as eigen-free Newton iteration in long double, started from
 // Tricomi's asymptotic estimate
@@ -72,18 +73,18 @@ int gs_quadrature_init(void)
     int dev = 0;
     GS_CHECK(cudaGetDevice(&dev));
     if (dev >= 0 && dev < 64 && g_gq_ready[dev]) return GS_OK;
-    static double t[GQ_VARIANTS][GQ_MAX], W[GQ_VARIANTS][GQ_MAX][4];
-    static float tf[GQ_VARIANTS][GQ_MAX], Wf[GQ_VARIANTS][GQ_MAX][4];
+    static double t[GQ_VARIANTS][GQ_MAX], W[GQ_VARIANTS][GQ_MAX][2];
+    static float tf[GQ_VARIANTS][GQ_MAX], Wf[GQ_VARIANTS][GQ_MAX][2];
     for (int v = 0; v < GQ_VARIANTS; v++) {
         long double tt[GQ_MAX], ww[GQ_MAX];
         int n = kGqN[v];
         gl_rule(n, tt, ww);
         for (int k = 0; k < GQ_MAX; k++) {
             long double x = k < n ? tt[k] : 0.0L, wk = k < n ? ww[k] : 0.0L;
-            long double L[4] = {1.0L, x, (3.0L * x * x - 1.0L) / 2.0L, (5.0L * x * x * x - 3.0L * x) / 2.0L};
+            long double L[2] = {1.0L, x};
             t[v][k] = (double)x;
             tf[v][k] = (float)x;
-            for (int j = 0; j < 4; j++) {
+            for (int j = 0; j < 2; j++) {
                 W[v][k][j] = (double)((2.0L * j + 1.0L) / 2.0L * wk * L[j]);
                 Wf[v][k][j] = (float)W[v][k][j];
             }
@@ -248,8 +249,8 @@ static int series_coeffs(double D, double hh, double R, double tol, const int *K
 static int gq_variant(double D, double hh, bool fp32)
 {
     const double a = sqrt(D) * hh;
-    if (fp32) return a <= 1.0 ? 0 : 2;   // 8 or 16 nodes
-    return a <= 0.25 ? 0 : (a <= 1.0 ? 2 : 3);   // 8, 16 or 24 nodes
+    if (fp32) return a <= 1.0 ? 0 : 1;   // 8 or 16 nodes
+    return a <= 0.25 ? 0 : (a <= 1.0 ? 1 : 2);   // 8, 16 or 24 nodes
 }
 
 // ---------------------------------------------------------------- octet geometry
@@ -593,7 +594,7 @@ static int grid_for(int64_t n_items, int per_block)
 }
 
 int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const uint8_t *d_vmask, int64_t n_oct,
-                 double *d_A, unsigned long long *d_pairs, unsigned *d_status, cudaStream_t st, cudaEvent_t *ev,
+                 double *d_A, unsigned long long *d_pairs, cudaStream_t st, cudaEvent_t *ev,
                  const GsProblem *d_probs, const int32_t *d_mol)
 {
     if (n_oct <= 0) return GS_OK;
@@ -619,18 +620,24 @@ int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const
     Series S;
     int K = 0;
     if (series_range64(P, hh)) K = series_coeffs(P.D, hh, P.pad, 1e-15, Ks, 7, &S);
-#define GS_ACC64(K_)                                                                                                    case K_: {                                                                                                              Series64<K_> c;                                                                                                     c.kappa = S.kappa;                                                                                                  for (int q = 0; q < 4; q++) memcpy(c.c[q], S.c[q], sizeof(double) * K_);                                            run(c);                                                                                                             break;                                                                                                          }
+#define GS_ACC64(K_)                                                                      \
+    case K_: {                                                                            \
+        Series64<K_> c;                                                                   \
+        c.kappa = S.kappa;                                                                \
+        for (int q = 0; q < 4; q++) memcpy(c.c[q], S.c[q], sizeof(double) * K_);          \
+        run(c);                                                                           \
+        break;                                                                            \
+    }
     switch (K) {
         GS_ACC64(7) GS_ACC64(8) GS_ACC64(9) GS_ACC64(10) GS_ACC64(12) GS_ACC64(15) GS_ACC64(20)
     default:
         switch (gq_variant(P.D, hh, false)) {
         case 0: run(Quad64<0, 8>()); break;
-        case 2: run(Quad64<2, 16>()); break;
-        default: run(Quad64<3, 24>()); break;
+        case 1: run(Quad64<1, 16>()); break;
+        default: run(Quad64<2, 24>()); break;
         }
     }
 #undef GS_ACC64
-    (void)d_status;
     if (ev) cudaEventRecord(ev[1], st);
     GS_CHECK(cudaGetLastError());
     return GS_OK;
@@ -651,9 +658,6 @@ __device__ __forceinline__ void load_tensor_f32(const float *__restrict__ src, f
 // Truncated SVD bounds of section 2.2.2: FP32 one thread per cube, FP64
 // (further down) four lanes or one warp per cube.
 
-template <typename T> __device__ __forceinline__ T t_sqrt(T x);
-template <> __device__ __forceinline__ double t_sqrt<double>(double x) { return sqrt(x); }
-template <> __device__ __forceinline__ float t_sqrt<float>(float x) { return sqrtf(x); }
 template <typename T> __device__ __forceinline__ T t_abs(T x) { return x < T(0) ? -x : x; }
 // Jacobi rotation zeroing the inner product ga of two rows with squared
 // norms al, be; false when the rows are already orthogonal to within 1e-6
@@ -684,20 +688,20 @@ __device__ __forceinline__ bool jac_rot(float al, float be, float ga, float &cs,
 // one-sided Jacobi on the 4 rows of X (4 x N): afterwards the rows are
 // orthogonal and X_in = Q^T X_out; sv receives their norms (the singular
 // values, unsorted)
-template <typename T, int N>
-__device__ __forceinline__ void jacobi_rows(T (&X)[4][N], T (&Q)[4][4], T (&sv)[4])
+template <int N>
+__device__ __forceinline__ void jacobi_rows(float (&X)[4][N], float (&Q)[4][4], float (&sv)[4])
 {
 #pragma unroll
     for (int a = 0; a < 4; a++)
 #pragma unroll
-        for (int b = 0; b < 4; b++) Q[a][b] = a == b ? T(1) : T(0);
+        for (int b = 0; b < 4; b++) Q[a][b] = a == b ? 1.f : 0.f;
     for (int sweep = 0; sweep < 40; sweep++) {
         bool any = false;
 #pragma unroll
         for (int p = 0; p < 3; p++)
 #pragma unroll
             for (int q = p + 1; q < 4; q++) {
-                T al = 0, be = 0, ga = 0;
+                float al = 0, be = 0, ga = 0;
                 {
                     // FP32: paired (f32x2) products over k = (2m, 2m+1), two
                     // partial sums each to shorten the dependency chains
@@ -716,7 +720,7 @@ __device__ __forceinline__ void jacobi_rows(T (&X)[4][N], T (&Q)[4][4], T (&sv)[
                     be = b.x + b.y;
                     ga = g.x + g.y;
                 }
-                T cs, sn;
+                float cs, sn;
                 if (!jac_rot(al, be, ga, cs, sn)) continue;
                 any = true;
                 {
@@ -745,24 +749,23 @@ __device__ __forceinline__ void jacobi_rows(T (&X)[4][N], T (&Q)[4][4], T (&sv)[
     }
 #pragma unroll
     for (int p = 0; p < 4; p++) {
-        T n2 = 0;
+        float n2 = 0;
 #pragma unroll
         for (int k = 0; k < N; k++) n2 += X[p][k] * X[p][k];
-        sv[p] = t_sqrt(n2);
+        sv[p] = sqrtf(n2);
     }
 }
 
 // the SVD of a 4 x 4 matrix: singular values sorted descending in s, the
 // matching left vectors in u, the right vectors (normalised rows) in X.  The
 // rows are sorted in place by a network of five exchanges.
-template <typename T>
-__device__ __forceinline__ void svd4(T (&X)[4][4], T (&s)[4], T (&u)[4][4])
+__device__ __forceinline__ void svd4(float (&X)[4][4], float (&s)[4], float (&u)[4][4])
 {
-    jacobi_rows<T, 4>(X, u, s);
+    jacobi_rows<4>(X, u, s);
     auto exchange = [&](int i, int j) {
         const bool sw = s[j] > s[i];
-        auto sel = [sw](T &p, T &q) {
-            const T a = sw ? q : p, b = sw ? p : q;
+        auto sel = [sw](float &p, float &q) {
+            const float a = sw ? q : p, b = sw ? p : q;
             p = a;
             q = b;
         };
@@ -780,7 +783,7 @@ __device__ __forceinline__ void svd4(T (&X)[4][4], T (&s)[4], T (&u)[4][4])
     exchange(1, 2);
 #pragma unroll
     for (int p = 0; p < 4; p++) {
-        const T inv = s[p] > T(0) ? T(1) / s[p] : T(0);
+        const float inv = s[p] > 0.f ? 1.f / s[p] : 0.f;
 #pragma unroll
         for (int k = 0; k < 4; k++) X[p][k] *= inv;
     }
@@ -841,23 +844,21 @@ __device__ __forceinline__ int rank99(const T (&s)[4], T &margin)
 // to the chosen one, and the one after it (if the chosen rule flipped, the
 // next one would decide).  RankNear records the rule nearest its threshold,
 // the rank it would give if it flipped, and the second-smallest distance.
-template <typename T>
 struct RankNear {
-    T m1, m2;      // smallest and second-smallest distance of a rule from its threshold
+    float m1, m2;      // smallest and second-smallest distance of a rule from its threshold
     int who;       // -1: outer rule; i >= 0: inner rule of kept term i
     int alt;       // rank that rule gives if it flips (0: none)
-    T ssum;        // sum of the outer singular values
+    float ssum;        // sum of the outer singular values
 };
 
-template <typename T>
-__device__ __forceinline__ void rank_near(const T (&s)[4], int r, int who, RankNear<T> &rn)
+__device__ __forceinline__ void rank_near(const float (&s)[4], int r, int who, RankNear &rn)
 {
-    T tot = s[0] + s[1] + s[2] + s[3];
-    T acc = 0;
-    T thr = T(0.99) * tot;
+    float tot = s[0] + s[1] + s[2] + s[3];
+    float acc = 0;
+    float thr = 0.99f * tot;
     for (int j = 0; j < 4 && j <= r; j++) {
         acc += s[j];
-        T m = t_abs(acc - thr);
+        float m = t_abs(acc - thr);
         // flipping rule j: below -> rank j+1; at or above -> the next rule decides
         int alt = acc >= thr ? j + 2 : j + 1;
         if (j == 3) alt = 0;
@@ -874,21 +875,20 @@ __device__ __forceinline__ void rank_near(const T (&s)[4], int r, int who, RankN
 
 // bounds: out = (L, U, sum|R|, sum|high|, rank, inner ranks); rmargin = the
 // smallest distance of a rank rule from its 99% threshold
-template <typename T>
-__device__ __forceinline__ T gap_sens(const T (&s)[4], int kept)
+__device__ __forceinline__ float gap_sens(const float (&s)[4], int kept)
 {
     // sum over the kept values of s_i / (distance to the nearest other
     // value): a perturbation E turns the i-th singular pair by about
     // |E| / gap_i, which moves that term's share of the bounds by about
     // s_i |E| / gap_i.  Terms far smaller than their gap contribute little.
-    T r = T(0);
+    float r = 0.f;
     for (int i = 0; i < kept && i < 4; i++) {
-        T g = T(1e30);
+        float g = 1e30f;
         if (i > 0) g = s[i - 1] - s[i];
-        if (i < 3) { T d = s[i] - s[i + 1]; g = d < g ? d : g; }
-        r += s[i] / (g > T(0) ? g : T(1e-30));
+        if (i < 3) { float d = s[i] - s[i + 1]; g = d < g ? d : g; }
+        r += s[i] / (g > 0.f ? g : 1e-30f);
     }
-    return r < T(1e6) ? r : T(1e6);
+    return r < 1e6f ? r : 1e6f;
 }
 
 // fo > 0 forces the outer rank; fi >= 0 forces the inner rank of kept term
@@ -901,9 +901,8 @@ __device__ __forceinline__ T gap_sens(const T (&s)[4], int kept)
 // FP64, took 53.4 ms: more instructions per cube than the paired FMAs here.
 #define EST_THREADS 128
 #define EST_SHARED 80
-template <typename T>
-__device__ __forceinline__ void estimate_bounds_sens(const T *A, T *S, T *out, T &rmargin, T &sens, int fo = 0, int fi = -1,
-                                                     int fj = 0, RankNear<T> *rn = nullptr);
+__device__ __forceinline__ void estimate_bounds_sens(const float *A, float *S, float *out, float &rmargin, float &sens, int fo = 0, int fi = -1,
+                                                     int fj = 0, RankNear *rn = nullptr);
 
 // element i of four (static indices only, so that arrays stay in registers)
 template <typename T>
@@ -915,14 +914,13 @@ __device__ __forceinline__ T sel4(int i, T a0, T a1, T a2, T a3)
 // The loops over kept terms are rolled, each term's row picked by static selects: one
 // copy of the inner SVD and bound code instead of one per possible rank,
 // which keeps the kernel within the instruction cache.
-template <typename T>
-__device__ __forceinline__ void estimate_bounds_sens(const T *A, T *S, T *out, T &rmargin, T &sens, int fo, int fi, int fj,
-                                                     RankNear<T> *rn)
+__device__ __forceinline__ void estimate_bounds_sens(const float *A, float *S, float *out, float &rmargin, float &sens, int fo, int fi, int fj,
+                                                     RankNear *rn)
 {
-    T s[4];
-    T high = 0, tot = 0;
+    float s[4];
+    float high = 0, tot = 0;
     {
-        T X[4][16], Q[4][4], sv[4];
+        float X[4][16], Q[4][4], sv[4];
         load_tensor_f32(A, &X[0][0]);
 #pragma unroll
         for (int j = 0; j < 4; j++)
@@ -932,18 +930,18 @@ __device__ __forceinline__ void estimate_bounds_sens(const T *A, T *S, T *out, T
                 if (j >= 2 || (k >> 2) >= 2 || (k & 3) >= 2) high += t_abs(X[j][k]);
             }
         out[3] = high;
-        rmargin = T(1e30);
-        sens = T(0);
-        if (tot == T(0)) { out[0] = out[1] = out[2] = 0; out[4] = 0; out[5] = 0; return; }
-        jacobi_rows<T, 16>(X, Q, sv);
+        rmargin = 1e30f;
+        sens = 0.f;
+        if (tot == 0.f) { out[0] = out[1] = out[2] = 0; out[4] = 0; out[5] = 0; return; }
+        jacobi_rows<16>(X, Q, sv);
         // row p goes to its place in descending order (equal values in row order)
 #pragma unroll
         for (int p = 0; p < 4; p++) {
             int pos = 0;
 #pragma unroll
             for (int q = 0; q < 4; q++) pos += (sv[q] > sv[p] || (sv[q] == sv[p] && q < p)) ? 1 : 0;
-            const T inv = sv[p] > T(0) ? T(1) / sv[p] : T(0);
-            T *row = S + 16 * pos * EST_THREADS, *left = S + (64 + 4 * pos) * EST_THREADS;
+            const float inv = sv[p] > 0.f ? 1.f / sv[p] : 0.f;
+            float *row = S + 16 * pos * EST_THREADS, *left = S + (64 + 4 * pos) * EST_THREADS;
 #pragma unroll
             for (int k = 0; k < 16; k++) row[k * EST_THREADS] = X[p][k] * inv;
 #pragma unroll
@@ -953,95 +951,95 @@ __device__ __forceinline__ void estimate_bounds_sens(const T *A, T *S, T *out, T
                 if (pos == i) s[i] = sv[p];
         }
     }
-    T rm;
+    float rm;
     int jr = rank99(s, rm);
     if (fo > 0) {
         jr = fo;
-        rm = T(1e30);
+        rm = 1e30f;
     } else if (rn) {
         rn->ssum = s[0] + s[1] + s[2] + s[3];
-        rank_near<T>(s, jr, -1, *rn);
+        rank_near(s, jr, -1, *rn);
     }
     rmargin = rm;
-    sens = gap_sens<T>(s, jr);
+    sens = gap_sens(s, jr);
     // R = A minus the kept rank-one terms, subtracted in place
-    T R[64];
+    float R[64];
     load_tensor_f32(A, R);
-    T M = 0, m = 0;
+    float M = 0, m = 0;
     int inner = 0;
 #pragma unroll 1
     for (int i = 0; i < jr; i++) {
-        T V[4][4], d[4], w[4][4], ui[4];
-        const T *row = S + 16 * i * EST_THREADS, *left = S + (64 + 4 * i) * EST_THREADS;
+        float V[4][4], d[4], w[4][4], ui[4];
+        const float *row = S + 16 * i * EST_THREADS, *left = S + (64 + 4 * i) * EST_THREADS;
 #pragma unroll
         for (int k = 0; k < 4; k++)
 #pragma unroll
             for (int l = 0; l < 4; l++) V[k][l] = row[(4 * k + l) * EST_THREADS];
 #pragma unroll
         for (int a = 0; a < 4; a++) ui[a] = left[a * EST_THREADS];
-        const T si0 = sel4(i, s[0], s[1], s[2], s[3]);
+        const float si0 = sel4(i, s[0], s[1], s[2], s[3]);
         svd4(V, d, w);
-        T rmi;
+        float rmi;
         int ji = rank99(d, rmi);
         if (i == fi) {
             ji = fj;
         } else {
             rmargin = rmi < rmargin ? rmi : rmargin;
-            if (rn) rank_near<T>(d, ji, i, *rn);
+            if (rn) rank_near(d, ji, i, *rn);
         }
-        T si = gap_sens<T>(d, ji);
+        float si = gap_sens(d, ji);
         sens = si > sens ? si : sens;
         inner += ji;
-        T Myz = 0, myz = 0;
+        float Myz = 0, myz = 0;
 #pragma unroll 1
         for (int k = 0; k < ji; k++) {
-            T wk[4], Vk[4];
+            float wk[4], Vk[4];
 #pragma unroll
             for (int b = 0; b < 4; b++) {
                 wk[b] = sel4(k, w[0][b], w[1][b], w[2][b], w[3][b]);
                 Vk[b] = sel4(k, V[0][b], V[1][b], V[2][b], V[3][b]);
             }
-            const T dk = sel4(k, d[0], d[1], d[2], d[3]);
-            T ly, hy, lz, hz;
+            const float dk = sel4(k, d[0], d[1], d[2], d[3]);
+            float ly, hy, lz, hz;
             cubic_range(wk, ly, hy);
             cubic_range(Vk, lz, hz);
-            T p0 = hy * hz, p1 = hy * lz, p2 = ly * hz, p3 = ly * lz;
-            T pmx = p0, pmn = p0;
+            float p0 = hy * hz, p1 = hy * lz, p2 = ly * hz, p3 = ly * lz;
+            float pmx = p0, pmn = p0;
             pmx = p1 > pmx ? p1 : pmx; pmn = p1 < pmn ? p1 : pmn;
             pmx = p2 > pmx ? p2 : pmx; pmn = p2 < pmn ? p2 : pmn;
             pmx = p3 > pmx ? p3 : pmx; pmn = p3 < pmn ? p3 : pmn;
             Myz += dk * pmx;
             myz += dk * pmn;
-            T sd = si0 * dk;
+            float sd = si0 * dk;
 #pragma unroll
             for (int a = 0; a < 4; a++) {
-                T sa = sd * ui[a];
+                float sa = sd * ui[a];
 #pragma unroll
                 for (int b = 0; b < 4; b++) {
-                    T sab = sa * wk[b];
+                    float sab = sa * wk[b];
 #pragma unroll
                     for (int cc = 0; cc < 4; cc++) R[16 * a + 4 * b + cc] -= sab * Vk[cc];
                 }
             }
         }
-        T lx, hx;
+        float lx, hx;
         cubic_range(ui, lx, hx);
-        T p0 = hx * Myz, p1 = hx * myz, p2 = lx * Myz, p3 = lx * myz;
-        T pmx = p0, pmn = p0;
+        float p0 = hx * Myz, p1 = hx * myz, p2 = lx * Myz, p3 = lx * myz;
+        float pmx = p0, pmn = p0;
         pmx = p1 > pmx ? p1 : pmx; pmn = p1 < pmn ? p1 : pmn;
         pmx = p2 > pmx ? p2 : pmx; pmn = p2 < pmn ? p2 : pmn;
         pmx = p3 > pmx ? p3 : pmx; pmn = p3 < pmn ? p3 : pmn;
         M += si0 * pmx;
         m += si0 * pmn;
     }
-    T sr = 0;
+    float sr = 0;
 #pragma unroll
     for (int t = 0; t < 64; t++) sr += t_abs(R[t]);
     out[0] = m - sr;
     out[1] = M + sr;
     out[2] = sr;
-    out[4] = (T)jr;
-    out[5] = (T)inner;
+    out[4] = (float)jr;
+    out[5] = (float)inner;
 }
 
 template <typename T>
@@ -2530,7 +2528,7 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 4) k_accum_f32(const __grid_co
 }
 
 int gs_accum_f32(const GsProblem &P, int level, const uint64_t *d_parents, const uint8_t *d_vmask, int64_t n_oct,
-                 float *d_A, float *d_err, unsigned long long *d_pairs, unsigned *d_status, cudaStream_t st, cudaEvent_t *ev,
+                 float *d_A, float *d_err, unsigned long long *d_pairs, cudaStream_t st, cudaEvent_t *ev,
                  unsigned long long *d_atom_octets, const GsProblem *d_probs, const int32_t *d_mol)
 {
     if (n_oct <= 0) return GS_OK;
@@ -2562,17 +2560,24 @@ int gs_accum_f32(const GsProblem &P, int level, const uint64_t *d_parents, const
     int K = 0;
     if (series_range32(P, hh)) K = series_coeffs(P.D, hh, P.pad, 2e-8, Ks, 5, &S);
     int rc;
-#define GS_ACC32(K_)                                                                                                    case K_: {                                                                                                              Series32<K_> c;                                                                                                     c.kappa = (float)S.kappa;                                                                                           for (int q = 0; q < 4; q++)                                                                                             for (int k = 0; k < K_; k++) c.c[q][k] = make_float2((float)S.c[q][k], (float)S.c[q][k]);                       rc = run("k_accum_f32<series" #K_ ">", c);                                                                         break;                                                                                                          }
+#define GS_ACC32(K_)                                                                                          \
+    case K_: {                                                                                                \
+        Series32<K_> c;                                                                                       \
+        c.kappa = (float)S.kappa;                                                                             \
+        for (int q = 0; q < 4; q++)                                                                           \
+            for (int k = 0; k < K_; k++) c.c[q][k] = make_float2((float)S.c[q][k], (float)S.c[q][k]);         \
+        rc = run("k_accum_f32<series" #K_ ">", c);                                                            \
+        break;                                                                                                \
+    }
     switch (K) {
         GS_ACC32(5) GS_ACC32(6) GS_ACC32(8) GS_ACC32(11) GS_ACC32(14)
     default:
         if (gq_variant(P.D, hh, true) == 0) rc = run("k_accum_f32<nodes8>", Quad32<0, 8>());
-        else rc = run("k_accum_f32<nodes16>", Quad32<2, 16>());
+        else rc = run("k_accum_f32<nodes16>", Quad32<1, 16>());
     }
 #undef GS_ACC32
     if (rc) return rc;
     if (ev) cudaEventRecord(ev[1], st);
-    (void)d_status;
     GS_CHECK(cudaGetLastError());
     return GS_OK;
 }
@@ -2699,9 +2704,9 @@ __device__ __forceinline__ void estimate_full_f32(const GsProblem &P, int level,
     }
     float b[6], rm;
     float sens;
-    RankNear<float> rn;
+    RankNear rn;
     rn.m1 = rn.m2 = 1e30f; rn.who = -1; rn.alt = 0; rn.ssum = 0.f;
-    estimate_bounds_sens<float>(A + q * 64, S, b, rm, sens, 0, -1, 0, &rn);
+    estimate_bounds_sens(A + q * 64, S, b, rm, sens, 0, -1, 0, &rn);
     const float c = (float)P.c, prec = (float)P.precision;
     int d = decide<float>(b, c, prec, level, P.max_depth);
     float dA = MIXED_KAPPA * E[q] + 1e-7f * tot;
@@ -2821,7 +2826,7 @@ __global__ void __launch_bounds__(EST_THREADS) k_estimate_alt(GsProblem P, int l
     const float c = (float)P.c, prec = (float)P.precision;
     const float dA = MIXED_KAPPA * E[q] + 1e-7f * tot;
     float b2[6], rm2, sens2;
-    estimate_bounds_sens<float>(A + q * 64, s_S + threadIdx.x, b2, rm2, sens2, who < 0 ? altr : 0, who, who < 0 ? 0 : altr, nullptr);
+    estimate_bounds_sens(A + q * 64, s_S + threadIdx.x, b2, rm2, sens2, who < 0 ? altr : 0, who, who < 0 ? 0 : altr, nullptr);
     const float bAlt = 4.f * (dA + 1e-7f * tot) * (1.f + fminf(sens2, 1e4f));
     const float mc2 = fminf(fabsf(c - b2[0]), fabsf(b2[1] - c));
     const bool ok = rm2 > 32.f * dA + 1e-5f * tot && decide<float>(b2, c, prec, level, P.max_depth) == (int)dec[q] &&
@@ -2954,7 +2959,8 @@ __global__ void k_count_mismatch(const uint8_t *a, const uint8_t *b, int64_t n, 
 // one chunk of a level in mixed precision; dec receives the final decisions
 // d_why: [0..2] flag reasons (bounds band, precision band, zero tensor), [3] low 32 bits = float bits of
 // the largest |A32 - A64| / E seen in debug mode, [4] the same for the band ratio, [5] flags through a rank
-// rule, [10] cubes decided without the SVD (corner values straddle c)
+// rule, [10] cubes decided without the SVD (corner values straddle c, range
+// and distance from rank one exclude it, or no atom reaches them)
 __global__ void k_gather_mol(const int64_t *__restrict__ si, int64_t m, const int32_t *__restrict__ mol,
                              int32_t *__restrict__ sub_mol)
 {
@@ -2964,7 +2970,7 @@ __global__ void k_gather_mol(const int64_t *__restrict__ si, int64_t m, const in
 
 int gs_level_mixed(const GsProblem &P, int level, const uint64_t *d_parents, int64_t n_oct, uint8_t *d_dec,
                    unsigned long long *d_pairs, unsigned long long *d_rechecked, unsigned long long *d_mism,
-                   bool both, unsigned *d_status, cudaStream_t st, cudaEvent_t *ev, unsigned long long *d_why,
+                   bool both, cudaStream_t st, cudaEvent_t *ev, unsigned long long *d_why,
                    const GsProblem *d_probs, const int32_t *d_mol, const uint8_t *d_vmask)
 {
     float *A = nullptr, *E = nullptr;
@@ -2976,7 +2982,7 @@ int gs_level_mixed(const GsProblem &P, int level, const uint64_t *d_parents, int
     if (!rc && both) rc = gs_alloc((void **)&dbg, sizeof(float) * 6 * 8 * (size_t)n_oct, st);
     // the counter block holds the atom-octet count 16 slots after the pair count
     if (!rc)
-        rc = gs_accum_f32(P, level, d_parents, d_vmask, n_oct, A, E, d_pairs, d_status, st, ev, d_pairs + 16, d_probs,
+        rc = gs_accum_f32(P, level, d_parents, d_vmask, n_oct, A, E, d_pairs, st, ev, d_pairs + 16, d_probs,
                           d_mol);
     if (!rc) rc = gs_estimate_f32(P, level, A, E, n_oct * 8, d_parents, d_vmask, d_dec, flag, st, d_why, dbg);
     if (!rc) {
@@ -3025,7 +3031,7 @@ int gs_level_mixed(const GsProblem &P, int level, const uint64_t *d_parents, int
                                                                                   sm);
             if (d_mol) GS_LAUNCH(k_gather_mol, (unsigned)((nsub + 255) / 256), 256, 0, st)(si, nsub, d_mol, smol);
             // only the flagged children are accumulated and estimated in FP64
-            rc = gs_accum_f64(P, level, sp, sm, nsub, A64, nullptr, d_status, st, nullptr, d_probs, smol);
+            rc = gs_accum_f64(P, level, sp, sm, nsub, A64, nullptr, st, nullptr, d_probs, smol);
         }
         int32_t *lst = nullptr;
         unsigned *nl = nullptr;
@@ -3051,7 +3057,7 @@ int gs_level_mixed(const GsProblem &P, int level, const uint64_t *d_parents, int
         if (!rc) rc = gs_alloc((void **)&b64, sizeof(double) * 6 * 8 * (size_t)n_oct, st);
         if (!rc) rc = gs_alloc((void **)&d64, 8 * (size_t)n_oct, st);
         if (!rc)
-            rc = gs_accum_f64(P, level, d_parents, d_vmask, n_oct, A64, nullptr, d_status, st, nullptr, d_probs, d_mol);
+            rc = gs_accum_f64(P, level, d_parents, d_vmask, n_oct, A64, nullptr, st, nullptr, d_probs, d_mol);
         if (!rc) rc = gs_estimate_f64(P, level, A64, n_oct * 8, d_parents, d_vmask, d64, b64, st);
         if (!rc) {
             unsigned nb = (unsigned)((n_oct * 8 + 255) / 256);
