@@ -1,15 +1,17 @@
-"""dL/dD for one atom far larger than the lattice spacing, where d^2 and r^2
+"""The adjoint at the ends of its range: dL/dD for one atom far larger than the lattice spacing, where d^2 and r^2
 nearly cancel in every term t (d^2 - r^2): against the same sum in numpy.
 
 All coordinates are multiples of 1/8, D is a power of two and D r^2 an
 integer, so d^2 - r^2 and the exponents are exact on both sides and a term's
-error is a few units of the exponentials' rounding."""
+error is a few units of the exponentials' rounding.  And atoms so far apart
+that the vertices are sorted into cells of twice the edge."""
 import math
 
 import numpy as np
 import pytest
 
 import oracle
+from meshcheck import key_normal_weights
 
 pytestmark = pytest.mark.gpu
 
@@ -43,3 +45,21 @@ def test_decay_rate_gradient():
     # per term: two exponentials of the field and one of the term, a division and eight products, about 16 roundings of
     # 1.1e-16, were they all to point one way (they do not: sums of 500,000 terms leave 1e-16)
     assert abs(gD - ref) <= 16 * 1.2e-16 * size
+
+
+def test_atoms_far_apart():
+    xyz = np.array([[0.0, 0.0, 0.0], [900.2, 910.1, 905.3], [450.1, 3.0, 880.2]])
+    r, D, h, depth = np.array([1.7, 1.2, 1.5]), 0.5, 0.5, 4
+    _, nroot, pad = oracle.root_grid(xyz, r, D, 1.0, h, depth)
+    # more than 2^24 cells of half the cutoff radius
+    assert np.prod(np.ceil(np.asarray(nroot) * h * 2.0 ** depth / (0.5 * pad)) + 1) > 1 << 24
+    m = gs.mesh_gaussian_surface(xyz, r, D, 1.0, 1e-3, depth, min_edge=h)
+    om = oracle.mesh(xyz, r, D, 1.0, 1e-3, h, depth)
+    assert np.array_equal(np.sort(m.vertex_keys), np.sort(om["vkeys"]))
+    ga, gr, gD = gs.gs_mesh_backward(xyz, r, D, 1.0, 1e-3, depth, key_normal_weights(m.vertex_keys), min_edge=h)
+    ox, orr, oD = oracle.mesh_grad(xyz, r, D, 1.0, 1e-3, h, depth, key_normal_weights(om["vkeys"]))
+    scale = max(np.abs(ox).max(), np.abs(orr).max(), abs(oD))
+    assert scale > 0.1
+    # the bar of the other adjoint tests
+    assert np.abs(ga - ox).max() <= 1e-9 * scale and np.abs(gr - orr).max() <= 1e-9 * scale
+    assert abs(gD - oD) <= 1e-9 * max(1.0, abs(oD))

@@ -2,7 +2,9 @@
 the same tensors whatever the number of octets in a launch (one warp per
 octet, or a block's four when there are few), the same bounds whatever the
 length of the list (one warp per cube, or four lanes in longer ones), and the same cubes in a
-batch as alone, also where a decision is a tie."""
+batch as alone, also where a decision is a tie; the same field at a point
+whatever the other points (a warp carries the last members of one point into
+the batches of the next)."""
 import numpy as np
 import pytest
 
@@ -103,3 +105,36 @@ def test_ties_in_a_batch(mode, which):
             assert b.stats[k] == one.stats[k], k
         assert np.array_equal(b.cube_keys, one.cube_keys)
         assert np.array_equal(b.vertices, one.vertices) and np.array_equal(b.triangles, one.triangles)
+
+
+def _points(n, seed):
+    """runs of points with no member, with a few and with more than 64"""
+    xyz, r = synth.globular(500, seed=40)
+    rng = np.random.default_rng(seed)
+    p = xyz[rng.integers(0, len(r), n)] + rng.normal(0, 1.0, (n, 3)) * rng.choice([0.5, 3.0, 12.0, 60.0], (n, 1))
+    p[100:400] += 500.0
+    return xyz, r, p
+
+
+@pytest.mark.parametrize("grad", [False, True])
+@pytest.mark.parametrize("n", [90001, 1300017])   # 2 and 32 points per warp, neither a multiple
+def test_field_of_a_set_and_its_parts(n, grad):
+    xyz, r, p = _points(n, seed=n)
+    whole = gs.gs_eval_field(xyz, r, D, C, p, grad=grad)
+    phi = whole[0] if grad else whole
+    assert (phi == 0).sum() > 300 and (phi > 0).sum() > n // 2
+    some = np.unique(np.concatenate([np.arange(0, n, 23), np.arange(90, 420), [n - 1]]))   # one point per warp
+    for take in (slice(0, 70003), slice(70003, n), some, np.random.default_rng(1).permutation(n)):
+        part = gs.gs_eval_field(xyz, r, D, C, np.ascontiguousarray(p[take]), grad=grad)
+        if grad:
+            assert np.array_equal(part[1], whole[1][take])
+            assert np.array_equal(part[0], phi[take])
+        else:
+            assert np.array_equal(part, phi[take])
+    assert np.array_equal(phi, gs.gs_eval_field(xyz, r, D, C, p))   # with and without the gradient
+    ref = oracle.field(xyz, r, D, C, p[some], grad=grad)
+    rphi = ref[0] if grad else ref
+    assert np.all(np.abs(phi[some] - rphi) <= 1e-13 * np.abs(rphi))
+    if grad:
+        # |dphi| <= 2 D R phi termwise
+        assert np.all(np.abs(whole[1][some] - ref[1]) <= 1e-12 * (np.abs(rphi)[:, None] + 1e-300) * 7.0)
