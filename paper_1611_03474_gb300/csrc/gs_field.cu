@@ -384,7 +384,11 @@ int gs_field_f64(const GsProblem &P, const uint64_t *d_vkeys, const double *d_po
 {
     if (n <= 0) return GS_OK;
     // one point per warp until there are 256 warps per SM (some eight times
-    // what is resident, for an even end), then up to 32
+    // what is resident, for an even end), then up to 32.  Calls at scattered
+    // points of 20,000 atoms with gradient, ms with 1, 8 and 32 points per warp
+    // and with this rule's number: 40,000: .55, .53, .61, .55 (1); 80,000: .87,
+    // .78, .86, .80 (2); 400,001: 3.31, 2.73, 2.77, 2.72 (10); 1,400,000: 10.96, 8.81,
+    // 8.65, 8.67 (32)
     const int64_t want = n / (152 * 256);
     const int ppw = (int)(want < 1 ? 1 : (want > 32 ? 32 : want));
     const int64_t nw = (n + ppw - 1) / ppw;
@@ -972,9 +976,12 @@ int gs_field_adjoint(const GsProblem &P, const int32_t *d_perm, const uint64_t *
             GS_LAUNCH(k_adj_starts, (unsigned)((nb + 256) / 256), 256, 0, st)(cnt, nb, starts);
             GS_LAUNCH(k_adj_scatter, gv, 256, 0, st)(V, d_vkeys, d_lambda, nv, cnt, vert, vertf);
             V.cell_start = starts;
-            // few atoms: several warps share one, until there are about 16 per SM
+            // few atoms: several warps share one, until there are about 32 per
+            // SM.  us with 1, 4, 8 and 16 warps per atom: 20 atoms: 244, 94, 66, 50; 200:
+            // 361, 166, 129, 121; 523: 391, 217, 206, 232; 1500: 645, 470, 453, 514; 2500: 758,
+            // 554, 551, 655 (670 with 2); 10,000: 1874, 1723, 1858, 2355
             const unsigned gx = (unsigned)((P.n + FD_WARPS - 1) / FD_WARPS);
-            const int64_t split = 152 * 16 / (P.n > 0 ? P.n : 1);
+            const int64_t split = P.n > 0 ? (152 * 32 + P.n - 1) / P.n : 1;
             const dim3 grid(gx, (unsigned)(split < 1 ? 1 : (split > 16 ? 16 : split)));
             GS_LAUNCH(k_field_adjoint, grid, 32 * FD_WARPS, 0, st)(V, d_perm, vert, vertf, d_gx, d_gr, d_gD);
         }

@@ -600,10 +600,12 @@ int gs_accum_f64(const GsProblem &P, int level, const uint64_t *d_parents, const
     if (n_oct <= 0) return GS_OK;
     const double hh = 0.5 * gs_h(P, level);
     if (ev) cudaEventRecord(ev[0], st);
-    // up to four blocks per SM.  One warp per octet against four (us), by octets
-    // listed: 153: 63 / 32; 281: 57 / 40; 362: 110 / 81; 575: 284 / 197; 1085:
-    // 61 / 106; 1139: 69 / 107; 2211: 206 / 255
-    const int split = n_oct <= 152 * 4 ? ACC_WARPS : 1;
+    // up to sixteen octets per SM.  One warp per octet against four (us), the
+    // last octets of the finest and of a coarser level of 20,000 atoms cut to
+    // length: 152: 124 / 45, 297 / 98; 608: 96 / 88, 233 / 167; 1216: 146 / 152,
+    // 396 / 319; 2432: 331 / 284, 752 / 661; 3648: 410 / 423, 1130 / 1026; 7296: 804 /
+    // 870, 2190 / 2141; 24,320: 2736 / 3097, 6973 / 7305
+    const int split = n_oct <= 152 * 16 ? ACC_WARPS : 1;
     const unsigned grid = grid_for(n_oct, ACC_WARPS / split);
     auto run = [&](auto coef) {
         using C = decltype(coef);
@@ -1474,9 +1476,11 @@ __device__ __forceinline__ void product_range(double l1, double h1, double l2, d
 }
 
 #define E64W_WARPS 4
-// the most cubes k_estimate_f64w takes: in FP64 meshes of 4 to 128 atoms it
-// took 55 us for 300 cubes, 73 for 840, 110 for 1475, 134 for 1914 and 227
-// for 3416; k_estimate_f64 141, 93, 154, 83 and 86
+// The most cubes k_estimate_f64w takes.  Its time grows by a step every 608
+// cubes (four warps per SM), that of k_estimate_f64 not before 4864.  The two
+// in us on lists of the finest and the coarsest level of 20,000 atoms cut to
+// length: 608: 47 / 88, 55 / 162; 1216: 69 / 90, 80 / 161; 1536: 98 / 92, 113 / 162; 2128:
+// 126 / 91, 149 / 162; 3040: 157 / 90, 186 / 163
 #define E64W_MAX 1536
 
 // the decision of cube q from its bounds, and the counts of small margins

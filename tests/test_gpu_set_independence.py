@@ -38,9 +38,9 @@ def _parts(xyz, r, keys, cuts):
 @pytest.mark.parametrize("atoms", [5, 600])
 def test_tensors_of_a_set_and_its_parts(level, atoms):
     xyz, r = synth.globular(atoms, seed=31)
-    keys = _keys(xyz, r, level, 700, seed=level)   # every key is an octet: more than four per SM
+    keys = _keys(xyz, r, level, 2600, seed=level)   # every key is an octet: more than sixteen per SM
     A, _, _ = gs.gs_cube_decisions(xyz, r, D, C, PREC, EDGE, DEPTH, keys)
-    Ap, _, _ = _parts(xyz, r, keys, (1, 90, 608))
+    Ap, _, _ = _parts(xyz, r, keys, (1, 150, 2582))
     assert np.abs(A).sum() > 0
     assert np.array_equal(A, Ap)
 
