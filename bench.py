@@ -4,9 +4,10 @@ a 250 A shell; D = 0.5, c = 1, precision 1e-3, min edge 0.25 A, 3 levels)
 on one GB300, through the C ABI.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--mode mixed|fp64]
-                  [--impl ours|reference]
+                  [--impl ours|reference] [--details FILE]
 
-One JSON line on rank 0.  `value` times mesh_gaussian_surface with the atoms
+One JSON line on rank 0 (under 3 KB; --details FILE writes the whole record,
+with every form's counts, stages and tuner choices).  `value` times mesh_gaussian_surface with the atoms
 already resident in HBM and the mesh left on the device; `e2e` times
 mesh_gaussian_surface_into with pinned host inputs and the mesh copied into
 pinned host buffers kept across calls, copies included.  L2
@@ -260,6 +261,30 @@ def readings_form(gs, synth, torch, dev, stream, steps, barrier):
     return out
 
 
+CONTRACT = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "gaussian_evals_per_s", "stage_ms", "clocks", "gpu_launches")
+
+
+def short_line(line):
+    """What the printed line keeps of the whole record: the contract's keys and
+    the headline figures of the other forms."""
+    out = {k: line[k] for k in CONTRACT if k in line}
+
+    def part(name, keys):
+        if line.get(name):
+            out[name] = {k: line[name][k] for k in keys if k in line[name]}
+
+    part("mesh", ("n_vertices", "n_triangles"))
+    part("roofline", ("bound", "kernel", "achieved", "peak", "unit", "frac", "ms_per_launch"))
+    part("e2e", ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "runs"))
+    part("fp64_form", ("ms_per_mesh", "same_cubes_and_topology", "max_vertex_diff_A"))
+    part("adaptive_form", ("ms_per_mesh", "n_triangles"))
+    part("diff_form", ("ms_forward", "ms_backward"))
+    part("batch_form", ("ms_per_batch", "ms_per_batch_threads", "ms_per_batch_sequential", "molecules_per_s"))
+    part("cpu_baseline", ("value", "unit", "cores", "kind", "extrapolated"))
+    return out
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -280,6 +305,7 @@ def main():
     ap.add_argument("--batch-steps", type=int, default=1, help="batch-form steps (64 molecules) to time")
     ap.add_argument("--readings-steps", type=int, default=1,
                     help="steps per alternative reading (20k atoms, FP64 form) timed and compared")
+    ap.add_argument("--details", metavar="FILE", help="write the whole record (JSON) to FILE")
     args = ap.parse_args()
     args.e2e_steps = max(1, args.e2e_steps)   # the line's e2e needs one measured call
     ws, rank, local = dist_env()
@@ -589,7 +615,10 @@ def main():
     if rank == 0 and ws == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline(cfg, examined_full=sum(st["examined"]))
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        if args.details:
+            with open(args.details, "w") as f:
+                json.dump(line, f)
+        print(json.dumps(short_line(line)), flush=True)
     if ws > 1:
         dist.destroy_process_group()
 
