@@ -2265,7 +2265,7 @@ struct Series32 {
 template <class C, bool BATCH>
 __global__ void __launch_bounds__(32 * ACC_WARPS, 4) k_accum_f32(const __grid_constant__ GsProblem P0, int level,
                                                                   const uint64_t *parents, const uint8_t *vmask,
-                                                                  int64_t n_oct, float hf, int lat_exact,
+                                                                  int64_t n_oct, float hf, float ctol, int lat_exact,
                                                                   const __grid_constant__ C coef,
                                                                   float *__restrict__ A_out,
                                                                   float *__restrict__ E_out,
@@ -2285,7 +2285,7 @@ __global__ void __launch_bounds__(32 * ACC_WARPS, 4) k_accum_f32(const __grid_co
     const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
     const int oWXY = ACF_WXY + ((cy * 2 + cx) * 4 + j) * 4, oZ = ACF_Z + 8 * cz;
     const float nDl2e = (float)(-P0.D * 1.4426950408889634);
-    const float hh = 0.5f * hf, ctol = fmaxf(1e-5f, 4e-7f * hf);
+    const float hh = 0.5f * hf;
     for (int64_t o = (int64_t)blockIdx.x * ACC_WARPS + wl; o < n_oct; o += (int64_t)gridDim.x * ACC_WARPS) {
         const GsProblem &P = BATCH ? probs[mol[o]] : P0;
         Octet q = octet_of(P, level, parents, vmask, o);
@@ -2537,6 +2537,7 @@ int gs_accum_f32(const GsProblem &P, int level, const uint64_t *d_parents, const
 {
     if (n_oct <= 0) return GS_OK;
     const double h = gs_h(P, level), hh = 0.5 * h;
+    const float ctol = fmaxf(1e-5f, 4e-7f * (float)h);   // the membership margin (see the kernel's filter)
     if (ev) cudaEventRecord(ev[0], st);
     // grid shapes the tuner chooses from: up to 64, 16 or 4 blocks per SM
     // (each warp takes every grid-th octet; the sums do not depend on it)
@@ -2551,11 +2552,11 @@ int gs_accum_f32(const GsProblem &P, int level, const uint64_t *d_parents, const
             unsigned long long *aoct = scratch ? (d_atom_octets ? scratch + 1 : nullptr) : d_atom_octets;
             if (d_probs)
                 GS_LAUNCH((k_accum_f32<C, true>), grid, 32 * ACC_WARPS, 0, st)(P, level, d_parents, d_vmask, n_oct,
-                                                                             (float)h, P.lat_exact_f32, coef, d_A,
+                                                                             (float)h, ctol, P.lat_exact_f32, coef, d_A,
                                                                              d_err, pairs, aoct, d_probs, d_mol);
             else
                 GS_LAUNCH((k_accum_f32<C, false>), grid, 32 * ACC_WARPS, 0, st)(P, level, d_parents, d_vmask, n_oct,
-                                                                              (float)h, P.lat_exact_f32, coef, d_A,
+                                                                              (float)h, ctol, P.lat_exact_f32, coef, d_A,
                                                                               d_err, pairs, aoct, nullptr, nullptr);
         });
     };
