@@ -128,9 +128,9 @@ typedef struct {
     int64_t recheck_rank;      /* mixed mode: of recheck_bounds, cubes flagged only through a rank rule near its threshold */
     int64_t vertex_mark_cubes[3]; /* mixed mode: surface cubes whose corners were re-evaluated in FP64 because the
                                      FP32 bound could move an edge point, flip a face saddle, move a fold root */
-    int64_t estimate_fast_cubes; /* mixed mode: cubes kept because the corner values of P~ straddle c, or discarded
-                                    because its range and its distance from rank one exclude c, decided
-                                    without the SVD bounds */
+    int64_t estimate_fast_cubes; /* mixed mode: cubes decided without the SVD bounds: kept because the corner values
+                                    of P~ straddle c, or discarded because no atom reaches them or because its
+                                    range and its distance from rank one exclude c */
     int64_t constrained_vertices; /* lattice vertices on a coarser cube's face or edge, whose value is that
                                      cube's interpolant (GS_CONFORM_CONSTRAIN) */
     int64_t agreement_splits;     /* cubes split because such an interpolant and the field value lay on
@@ -141,7 +141,8 @@ typedef struct {
     int64_t near_threshold[4];    /* decisions taken in FP64 whose margin was below 1e-10 relative: [0] bound
                                      test, min(c-L, U-c) against |c|+|L|+|U|; [1] precision test, |precision -
                                      sum|high|| against their sum; [2] a 99% rank rule, |sum_{i<=j} s_i - 0.99
-                                     sum s| against sum s; [3] lattice vertices with |value - c| < 1e-10 c.  Such
+                                     sum s| against sum s (of the cubes whose SVD was taken: a cube decided without
+                                     it holds for any ranks); [3] lattice vertices with |value - c| < 1e-10 c.  Such
                                      a decision may differ from an independent FP64 evaluation by rounding
                                      alone (the oracle resolves them in quad precision) */
     int64_t refine_vertices;      /* mixed mode: lattice vertex values re-evaluated in double-word FP32 (a hi + lo

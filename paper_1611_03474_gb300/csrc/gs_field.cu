@@ -815,7 +815,7 @@ int gs_field_refine(const GsProblem &P, const uint64_t *d_vkeys, int64_t n, int6
 // a queue of members as in k_field_f64, and adds its five sums to the
 // gradient once.  With one thread per vertex every term cost four FP64
 // atomics and most lanes of an FP64 instruction were empty (10,000 atoms,
-// 43.7M terms: 4.53 ms; 1.66 ms and 0.09 ms for the sorting).
+// 43.7M terms: 4.53 ms; 1.7 ms and 0.09 ms for the sorting).
 
 // the grid the vertices are sorted into: V.cell_f, V.cdim and V.cell_start of
 // a copy of the problem, for gs_warp_candidates
