@@ -1532,7 +1532,9 @@ static int batch_shared(const double *atoms, const double *radii, const int64_t 
         }
         // one level loop per coefficient class, so that each molecule's tensors
         // are those of its own call (nearly always one class: cubes of 2 to 0.25
-        // A at D = 0.5 have one for largest radii of 1.5 to 1.8 A)
+        // A at D = 0.5 have one for largest radii of 1.5 to 1.8 A).  More classes
+        // cost more launches: 16 molecules with radii scaled by 0.7 to 1.6 each take
+        // 34 ms instead of 29, on one stream or on four.
         std::vector<std::vector<int>> classes;
         std::vector<std::vector<int64_t>> parts;
         if (!rc)

@@ -27,7 +27,12 @@ def _grid(n):
     rng = np.random.default_rng(n)
     vals = rng.standard_normal((n, n, n))
     vals[0], vals[-1], vals[:, 0], vals[:, -1], vals[:, :, 0], vals[:, :, -1] = -1, -1, -1, -1, -1, -1
-    return gs.gs_triangulate_grid(vals, 0.0)
+    m = gs.gs_triangulate_grid(vals, 0.0)
+    c = [slice(0, n - 1), slice(1, n)]
+    inside = np.stack([vals[i, j, k] > 0 for i in c for j in c for k in c])
+    surface = (inside.any(axis=0) & ~inside.all(axis=0)).sum()
+    assert len(m.triangles) > 4 * surface   # so some cubes overflow their slot of four
+    return m
 
 
 def _mixed_sizes():
